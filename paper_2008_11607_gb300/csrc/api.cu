@@ -57,6 +57,7 @@ struct rexi_plan_s {
   int shift_mode = REXI_SHIFT_NONE;
   double shift_value = 0.0;  // sigma requested with REXI_SHIFT_VALUE
   double sigma = 0.0;        // sigma in effect (scalar operator only)
+  double lambda_min = 0.0;   // smallest eigenvalue of d_xx + d_yy (the largest is 0; scalar operator only)
   double Hmax = 0.0, Hmean = 0.0;
   // Fourier path tables (device)
   FftPlan1D fx, fy;
@@ -75,6 +76,7 @@ struct rexi_plan_s {
   float4* halfdf_y = nullptr;
   double2* half_x = nullptr;
   double2* half_y = nullptr;
+  double* cell_tab = nullptr;  // tables of the local-expansion pole sum (cell_tables_host)
   // device coefficient tables of the FP64 and mixed Fourier forms, one per
   // (form, M, term range, split grid); immutable once uploaded
   struct CoefTable {
@@ -126,6 +128,19 @@ void prof_mark(rexi_plan_s* p, int i, cudaStream_t s) {
   cudaEventRecord(p->prof_pool[p->prof_used - 1][i], s);
 }
 }  // namespace
+
+template <typename T>
+static bool upload_table(const std::vector<T>& host, T** dev, rexi_status* st) {
+  if (cudaMalloc(dev, host.size() * sizeof(T)) != cudaSuccess) {
+    *st = fail(REXI_ENOMEM, "cudaMalloc of a plan table failed");
+    return false;
+  }
+  if (cudaMemcpy(*dev, host.data(), host.size() * sizeof(T), cudaMemcpyHostToDevice) != cudaSuccess) {
+    *st = fail(REXI_ECUDA, "upload of a plan table failed");
+    return false;
+  }
+  return true;
+}
 
 extern "C" {
 
@@ -237,6 +252,7 @@ void rexi_plan_destroy(rexi_plan_t p) {
   cudaFree(p->halfdf_y);
   cudaFree(p->half_x);
   cudaFree(p->half_y);
+  cudaFree(p->cell_tab);
   if (p->staging) cudaFreeHost(p->staging);
   for (auto& c : p->coef) {
     cudaFree(c.dev);
@@ -247,18 +263,6 @@ void rexi_plan_destroy(rexi_plan_t p) {
   for (auto& set : p->prof_pool)
     for (auto e : set) cudaEventDestroy(e);
   delete p;
-}
-
-static bool upload_table(const std::vector<double2>& host, double2** dev, rexi_status* st) {
-  if (cudaMalloc(dev, host.size() * sizeof(double2)) != cudaSuccess) {
-    *st = fail(REXI_ENOMEM, "cudaMalloc of a plan table failed");
-    return false;
-  }
-  if (cudaMemcpy(*dev, host.data(), host.size() * sizeof(double2), cudaMemcpyHostToDevice) != cudaSuccess) {
-    *st = fail(REXI_ECUDA, "upload of a plan table failed");
-    return false;
-  }
-  return true;
 }
 
 rexi_status rexi_plan_create(rexi_plan_t* out, int32_t nx, int32_t ny, double Lx, double Ly, double g,
@@ -297,7 +301,8 @@ rexi_status rexi_plan_create(rexi_plan_t* out, int32_t nx, int32_t ny, double Lx
     make(nx, twx, hx);
     make(ny, twy, hy);
     if (!upload_table(twx, &p->tw_x, &st) || !upload_table(twy, &p->tw_y, &st) ||
-        !upload_table(hx, &p->half_x, &st) || !upload_table(hy, &p->half_y, &st)) {
+        !upload_table(hx, &p->half_x, &st) || !upload_table(hy, &p->half_y, &st) ||
+        !upload_table(cell_tables_host(), &p->cell_tab, &st)) {
       rexi_plan_destroy(p);
       return st;
     }
@@ -738,34 +743,51 @@ rexi_status fourier_step(rexi_plan_s* p, const void* in, void* out, double dt, i
     if (half) fs.R0im = 0.0;
     const int row_len = half ? p->nx / 2 + 1 : p->nx;
     const OrbitParams op = orbit_params(sp);
-    const int slices = pole_orbit_slices(p->form, op.norb, fs.nterms, L.slice_cap);
     double2* part = reinterpret_cast<double2*>(base + L.part_off);
+    void* fin = base + L.fin_off;
+    // the combine of complex input in the mixed form takes the FP64 scalars
+    const OrbitOut kind = p->spectral == 2 ? kOrbitRaw : df_spec ? kOrbitDf : kOrbitFp64;
+    // range of x = tau omega over the grid's wavenumbers (signed for the scalar operator)
+    const double x_lo = p->spectral == 2 ? tau * (p->lambda_min - p->sigma) : 0.0;
+    const double x_hi = tau * (p->spectral == 2 ? -p->sigma : p->rho_natural);
+    CellGeom cg;
+    const bool cells = cell_geometry(p->form, op.norb, fs.nterms, tb, te, h, q, x_lo, x_hi, G, &cg) &&
+                       cell_scratch_values(cg) <= (size_t)L.slice_cap * op.norb;
+    const void* raw = fin;  // kOrbitRaw: R+ of every orbit, as raw_slices partial sums
+    int raw_slices = 1;
     if ((st = forward()) != REXI_OK) return st;
-    if (p->form == REXI_FORM_FP64)
-      CUDA_TRY(pole_orbits_fp64(part, slices, sp, op, static_cast<const double*>(ct->dev), fs, s),
-               "pole_orbits_fp64");
-    else
-      CUDA_TRY(pole_orbits_mixed(part, slices, sp, op, static_cast<const float*>(ct->dev), fs, G, s),
-               "pole_orbits_mixed");
+    if (cells) {
+      CUDA_TRY(pole_cells(p->form, cg, cell_tables_at(p->cell_tab), ct->dev, part, sp, op, fs, kind, fin, s),
+               "pole_cells");
+      p->launches += cg.two_level ? 2 : 1;
+    } else {
+      const int slices = pole_orbit_slices(p->form, op.norb, fs.nterms, L.slice_cap);
+      if (p->form == REXI_FORM_FP64)
+        CUDA_TRY(pole_orbits_fp64(part, slices, sp, op, static_cast<const double*>(ct->dev), fs, s),
+                 "pole_orbits_fp64");
+      else
+        CUDA_TRY(pole_orbits_mixed(part, slices, sp, op, static_cast<const float*>(ct->dev), fs, G, s),
+                 "pole_orbits_mixed");
+      if (kind != kOrbitRaw)  // the scalar combine sums the slices itself
+        CUDA_TRY(pole_orbit_finalize(part, slices, sp, op, fs, kind, fin, s), "pole_orbit_finalize");
+      raw = part;
+      raw_slices = slices;
+    }
     prof_mark(p, 5, s);
     if (p->spectral == 2) {
       // e^{tau A} = e^{i tau sigma} e^{tau (A - i sigma I)}
       const double2 phase = make_double2(cos(tau * p->sigma), sin(tau * p->sigma));
-      CUDA_TRY(pole_orbit_combine_scalar(spec, part, slices, sp, op, phase, adjoint ? 1 : 0, s),
+      CUDA_TRY(pole_orbit_combine_scalar(spec, raw, raw_slices, sp, op, phase, adjoint ? 1 : 0, s),
                "pole_orbit_combine_scalar");
     } else if (p->form == REXI_FORM_MIXED && !half && !p->spectral) {
       // complex input (or real input without the half-length transform): the
       // combine in double-float arithmetic on the FP64 spectrum
-      CUDA_TRY(pole_orbit_combine_dfc(spec, part, slices, base + L.fin_off, sp, p->halfdf_x, p->halfdf_y, op, fs,
-                                      s),
-               "pole_orbit_combine_dfc");
+      CUDA_TRY(pole_orbit_combine_dfc(spec, fin, sp, p->halfdf_x, p->halfdf_y, op, fs, s), "pole_orbit_combine_dfc");
     } else if (df_spec)
-      CUDA_TRY(pole_orbit_combine_df(spec, part, slices, base + L.fin_off, sp, p->halfdf_x, p->halfdf_y, op, fs,
-                                     row_len, s),
+      CUDA_TRY(pole_orbit_combine_df(spec, fin, sp, p->halfdf_x, p->halfdf_y, op, fs, row_len, s),
                "pole_orbit_combine_df");
     else
-      CUDA_TRY(pole_orbit_combine(spec, part, slices, base + L.fin_off, sp, op, fs, row_len, s),
-               "pole_orbit_combine");
+      CUDA_TRY(pole_orbit_combine(spec, fin, sp, op, fs, row_len, s), "pole_orbit_combine");
     p->launches += 3;
   } else {
     // plain form: terms n = 0..N (real) or -N..N (complex), |n| in [tb, te)
@@ -1045,6 +1067,7 @@ void update_rho(rexi_plan_s* p) {
     p->sigma = p->shift_mode == REXI_SHIFT_MIDPOINT ? 0.5 * (lmin + lmax)
                : p->shift_mode == REXI_SHIFT_VALUE  ? p->shift_value
                                                     : 0.0;
+    p->lambda_min = lmin;
     p->rho = p->rho_natural = std::max(fabs(lmin - p->sigma), fabs(lmax - p->sigma));
   } else {
     p->sigma = 0.0;

@@ -685,12 +685,14 @@ rexi_status rexi_batch_step(rexi_batch_t b, const void* in, void* out, int32_t r
                 ? pole_orbits_fp64(part, slices, sp, op, reinterpret_cast<const double*>(tab), fs, s)
                 : pole_orbits_mixed(part, slices, sp, op, tab, fs, D.grid, s);
       void* fin = orb + per_instance_part_bytes(D);
+      if (e == cudaSuccess)
+        e = pole_orbit_finalize(part, slices, sp, op, fs, half && df ? kOrbitDf : kOrbitFp64, fin, s);
       const double scale = 1.0 / ((double)D.nx * D.ny);
       if (e == cudaSuccess) {
         if (half && df)
-          e = pole_orbit_combine_df(sp_i, part, slices, fin, sp, D.halfdf_x, D.halfdf_y, op, fs, D.nx / 2 + 1, s);
+          e = pole_orbit_combine_df(sp_i, fin, sp, D.halfdf_x, D.halfdf_y, op, fs, D.nx / 2 + 1, s);
         else
-          e = pole_orbit_combine(sp_i, part, slices, fin, sp, op, fs, half ? D.nx / 2 + 1 : D.nx, s);
+          e = pole_orbit_combine(sp_i, fin, sp, op, fs, half ? D.nx / 2 + 1 : D.nx, s);
       }
       if (e == cudaSuccess)
         e = half ? fft2d_c2r(sp_i, out2 + D.spec_off, 3, fx, fxh, fy, scale, df, s)

@@ -128,31 +128,62 @@ cudaError_t pole_orbits_fp64(double2* part, int slices, const SymbolParams& sp, 
                              const double* table, const FusedScalars& fs, cudaStream_t s);
 cudaError_t pole_orbits_mixed(double2* part, int slices, const SymbolParams& sp, const OrbitParams& op,
                               const float* table, const FusedScalars& fs, double grid, cudaStream_t s);
-// spec <- r(tau B) spec at every wavenumber, R+ = sum over slices of part:
-// a per-orbit pass writes the combine scalars to `fin`
-// (orbit_scalars_bytes(norb) bytes, 32-byte aligned), then a pass over the
-// wavenumbers applies them.  row_len: nx (full spectrum, rows of nx values)
-// or nx/2 + 1 (half spectrum of real input, wavenumbers kx = 0..nx/2 only).
-cudaError_t pole_orbit_combine(double2* spec, const double2* part, int slices, void* fin, const SymbolParams& sp,
-                               const OrbitParams& op, const FusedScalars& fs, int row_len, cudaStream_t s);
+// What a pole sum leaves per orbit in `fin` (orbit_scalars_bytes(norb) bytes,
+// 32-byte aligned): the combine scalars of r(tau B) in FP64, the same as
+// double-float pairs of the real s1 and s2 (real R0), or R+ itself (double2,
+// from pole_cells only).
+enum OrbitOut { kOrbitFp64 = 0, kOrbitDf = 1, kOrbitRaw = 2 };
 size_t orbit_scalars_bytes(int norb);
+// fin from the sum over slices of part.
+cudaError_t pole_orbit_finalize(const double2* part, int slices, const SymbolParams& sp, const OrbitParams& op,
+                                const FusedScalars& fs, OrbitOut kind, void* fin, cudaStream_t s);
+
+// ---- pole sums by local expansion (pole_cells.cu, pole_cells.cuh) ----------
+constexpr int kCellP = 16;   // nodes per cell
+constexpr int kCellK = 32;   // cells per coarse cell
+constexpr int kCellPC = 24;  // nodes per coarse cell
+struct CellGeom {
+  double c, w, inv_c, inv_w, inv_h, q, grid, inv_grid;  // c: half-width of a cell (a power of two), w = 2c
+  float q_hi, q_lo;
+  int k0, ncell, ncoarse, two_level;  // cells k0 .. k0 + ncell - 1, cell k on [k w, (k + 1) w)
+  int tb, te, nterms;                 // the table's terms: |n| in [tb, te), n ascending
+};
+struct CellTables {  // device tables, the same for every plan (cell_tables_host)
+  const double *node_t, *coarse_t, *spread, *to_cheb, *to_mono;
+};
+const std::vector<double>& cell_tables_host();
+CellTables cell_tables_at(const double* dev);
+// The cells for x in [x_lo, x_hi], or false where summing every orbit directly costs less.
+bool cell_geometry(int form, int norb, int nterms, int tb, int te, double h, double q, double x_lo, double x_hi,
+                   double grid, CellGeom* g);
+size_t cell_scratch_values(const CellGeom& g);  // double2 values of scratch
+// fin of every orbit, as pole_orbits_* and pole_orbit_finalize leave it.
+cudaError_t pole_cells(int form, const CellGeom& g, const CellTables& T, const void* table, double2* scratch,
+                       const SymbolParams& sp, const OrbitParams& op, const FusedScalars& fs, OrbitOut kind,
+                       void* fin, cudaStream_t s);
+
+// spec <- r(tau B) spec at every wavenumber from the orbits' scalars.
+// row_len: nx (full spectrum, rows of nx values) or nx/2 + 1 (half spectrum
+// of real input, wavenumbers kx = 0..nx/2 only).
+cudaError_t pole_orbit_combine(double2* spec, const void* fin, const SymbolParams& sp, const OrbitParams& op,
+                               const FusedScalars& fs, int row_len, cudaStream_t s);
 // The same on a half spectrum kept as double-float pairs (float4 per value),
 // in double-float arithmetic; C-grid symbol and real R0 (real input) only,
 // cudaErrorInvalidValue otherwise.  half_x_df, half_y_df: (cos, sin) of
 // pi k / n as double-float pairs.
 // Complex input in the mixed form (C grid): the combine of pole_orbit_combine
 // (full spectrum, FP64 storage) in double-float arithmetic.
-cudaError_t pole_orbit_combine_dfc(double2* spec, const double2* part, int slices, void* fin, const SymbolParams& sp,
-                                   const float4* half_x_df, const float4* half_y_df, const OrbitParams& op,
-                                   const FusedScalars& fs, cudaStream_t s);
+cudaError_t pole_orbit_combine_dfc(double2* spec, const void* fin, const SymbolParams& sp, const float4* half_x_df,
+                                   const float4* half_y_df, const OrbitParams& op, const FusedScalars& fs,
+                                   cudaStream_t s);
 // Scalar operators (SymbolParams::spectral == 2): spec <- phase R(k) spec on
-// every field of the full spectrum (rows of nx values), R the sum over slices
-// of the orbit's partial sums; conj(phase R) for the adjoint.
-cudaError_t pole_orbit_combine_scalar(double2* spec, const double2* part, int slices, const SymbolParams& sp,
+// every field of the full spectrum (rows of nx values), R the sum of `slices`
+// partial sums per orbit (double2); conj(phase R) for the adjoint.
+cudaError_t pole_orbit_combine_scalar(double2* spec, const void* part, int slices, const SymbolParams& sp,
                                       const OrbitParams& op, double2 phase, int adjoint, cudaStream_t s);
-cudaError_t pole_orbit_combine_df(void* spec_df, const double2* part, int slices, void* fin, const SymbolParams& sp,
-                                  const float4* half_x_df, const float4* half_y_df, const OrbitParams& op,
-                                  const FusedScalars& fs, int row_len, cudaStream_t s);
+cudaError_t pole_orbit_combine_df(void* spec_df, const void* fin, const SymbolParams& sp, const float4* half_x_df,
+                                  const float4* half_y_df, const OrbitParams& op, const FusedScalars& fs, int row_len,
+                                  cudaStream_t s);
 struct PlainScalars {
   double tau;
   int nterms;   // terms in this chunk

@@ -142,6 +142,34 @@ __device__ __forceinline__ OrbitScalars orbit_scalars(double omega, double2 R0, 
   return o;
 }
 
+// The real s1 and s2 as double-float pairs for the double-float combine.
+struct OrbitScalarsDF {
+  float2 s1, s2;
+};
+
+__device__ __forceinline__ float2 df_split(double v) {
+  const float h = (float)v;
+  return make_float2(h, (float)(v - (double)h));
+}
+
+// fin[o] from R+ of orbit o (see OrbitOut).
+template <int KIND>
+__device__ __forceinline__ void orbit_store(void* fin, int o, double omega, double2 R0, double2 Rp) {
+  if (KIND == kOrbitRaw) {
+    static_cast<double2*>(fin)[o] = Rp;
+    return;
+  }
+  const OrbitScalars sc = orbit_scalars(omega, R0, Rp);
+  if (KIND == kOrbitDf) {
+    OrbitScalarsDF d;
+    d.s1 = df_split(sc.s1);
+    d.s2 = df_split(sc.s2re);
+    static_cast<OrbitScalarsDF*>(fin)[o] = d;
+  } else {
+    static_cast<OrbitScalars*>(fin)[o] = sc;
+  }
+}
+
 // The six nonzero entries of B(k) with g, H and f folded in (or of B^H for
 // the adjoint: (B^H)_ij = conj(B_ji)):
 //   y0 = e01 f1 + e02 f2,  y1 = e10 f0 + e12 f2,  y2 = e20 f0 + e21 f1.

@@ -179,19 +179,9 @@ __global__ void __launch_bounds__(kOrbitThreads) pole_orbit_mixed_kernel(double2
           make_double2((double)ar_h[u] + (double)ar_l[u], (double)ai_h[u] + (double)ai_l[u]);
 }
 
-// Per orbit: R+ = sum of the slices' partial sums (fixed order), then the
-// combine scalars at the representative's omega (FP64, or double-float pairs
-// of the real s1 and s2 for the double-float combine, where R0 is real).
-struct OrbitScalarsDF {
-  float2 s1, s2;
-};
-
-__device__ __forceinline__ float2 df_split(double v) {
-  const float h = (float)v;
-  return make_float2(h, (float)(v - (double)h));
-}
-
-template <bool DF>
+// Per orbit: R+ = sum of the slices' partial sums (fixed order), then what
+// the combine pass takes, at the representative's omega (see OrbitOut).
+template <int KIND>
 __global__ void __launch_bounds__(256) pole_orbit_finalize_kernel(const double2* __restrict__ part, int slices,
                                                                   SymbolParams sp, OrbitParams op, double2 R0,
                                                                   void* __restrict__ fin) {
@@ -205,15 +195,7 @@ __global__ void __launch_bounds__(256) pole_orbit_finalize_kernel(const double2*
   }
   int a, b;
   orbit_rep(op, o, a, b);
-  const OrbitScalars sc = orbit_scalars(symbol_at(sp, a, b).omega, R0, Rp);
-  if (DF) {
-    OrbitScalarsDF d;
-    d.s1 = df_split(sc.s1);
-    d.s2 = df_split(sc.s2re);
-    static_cast<OrbitScalarsDF*>(fin)[o] = d;
-  } else {
-    static_cast<OrbitScalars*>(fin)[o] = sc;
-  }
+  orbit_store<KIND>(fin, o, symbol_at(sp, a, b).omega, R0, Rp);
 }
 
 __global__ void __launch_bounds__(256) pole_orbit_combine_kernel(double2* spec,
@@ -309,15 +291,19 @@ cudaError_t pole_orbits_mixed(double2* part, int slices, const SymbolParams& sp,
   return cudaGetLastError();
 }
 
-cudaError_t pole_orbit_combine(double2* spec, const double2* part, int slices, void* fin, const SymbolParams& sp,
-                               const OrbitParams& op, const FusedScalars& fs, int row_len, cudaStream_t s) {
+cudaError_t pole_orbit_finalize(const double2* part, int slices, const SymbolParams& sp, const OrbitParams& op,
+                                const FusedScalars& fs, OrbitOut kind, void* fin, cudaStream_t s) {
   const double2 R0 = make_double2(fs.R0re, fs.R0im);
-  OrbitScalars* F = static_cast<OrbitScalars*>(fin);
-  pole_orbit_finalize_kernel<false><<<(unsigned)((op.norb + 255) / 256), 256, 0, s>>>(part, slices, sp, op, R0, F);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  auto k = kind == kOrbitDf ? pole_orbit_finalize_kernel<kOrbitDf> : pole_orbit_finalize_kernel<kOrbitFp64>;
+  k<<<(unsigned)((op.norb + 255) / 256), 256, 0, s>>>(part, slices, sp, op, R0, fin);
+  return cudaGetLastError();
+}
+
+cudaError_t pole_orbit_combine(double2* spec, const void* fin, const SymbolParams& sp, const OrbitParams& op,
+                               const FusedScalars& fs, int row_len, cudaStream_t s) {
   const size_t nk = (size_t)row_len * sp.ny;
-  pole_orbit_combine_kernel<<<(unsigned)((nk + 255) / 256), 256, 0, s>>>(spec, F, sp, op, R0, fs.adjoint, row_len);
+  pole_orbit_combine_kernel<<<(unsigned)((nk + 255) / 256), 256, 0, s>>>(
+      spec, static_cast<const OrbitScalars*>(fin), sp, op, make_double2(fs.R0re, fs.R0im), fs.adjoint, row_len);
   return cudaGetLastError();
 }
 
@@ -337,15 +323,10 @@ __global__ void __launch_bounds__(256) pole_orbit_combine_dfc_kernel(double2* sp
   combine_dfc_at(spec, k, nk, kx, ky, sd, c0, df_from_double(o.s1), s2, adjoint != 0);
 }
 
-cudaError_t pole_orbit_combine_dfc(double2* spec, const double2* part, int slices, void* fin, const SymbolParams& sp,
-                                   const float4* half_x_df, const float4* half_y_df, const OrbitParams& op,
-                                   const FusedScalars& fs, cudaStream_t s) {
+cudaError_t pole_orbit_combine_dfc(double2* spec, const void* fin, const SymbolParams& sp, const float4* half_x_df,
+                                   const float4* half_y_df, const OrbitParams& op, const FusedScalars& fs,
+                                   cudaStream_t s) {
   if (sp.spectral) return cudaErrorInvalidValue;  // the C grid only
-  const double2 R0 = make_double2(fs.R0re, fs.R0im);
-  OrbitScalars* F = static_cast<OrbitScalars*>(fin);
-  pole_orbit_finalize_kernel<false><<<(unsigned)((op.norb + 255) / 256), 256, 0, s>>>(part, slices, sp, op, R0, F);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
   SymbolDF sd;
   sd.g = df_split_host(sp.g);
   sd.H = df_split_host(sp.H);
@@ -357,8 +338,8 @@ cudaError_t pole_orbit_combine_dfc(double2* spec, const double2* part, int slice
   const float2 c0r = df_split_host(fs.R0re), c0i = df_split_host(fs.adjoint ? -fs.R0im : fs.R0im);
   const float4 c0 = make_float4(c0r.x, c0r.y, c0i.x, c0i.y);
   const size_t nk = (size_t)sp.nx * sp.ny;
-  pole_orbit_combine_dfc_kernel<<<(unsigned)((nk + 255) / 256), 256, 0, s>>>(spec, F, sd, sp.nx, sp.ny, op, c0,
-                                                                             fs.adjoint);
+  pole_orbit_combine_dfc_kernel<<<(unsigned)((nk + 255) / 256), 256, 0, s>>>(
+      spec, static_cast<const OrbitScalars*>(fin), sd, sp.nx, sp.ny, op, c0, fs.adjoint);
   return cudaGetLastError();
 }
 
@@ -384,23 +365,19 @@ __global__ void __launch_bounds__(256) pole_orbit_combine_scalar_kernel(double2*
   for (int c = 0; c < 3; ++c) spec[k + c * nk] = cm(m, spec[k + c * nk]);
 }
 
-cudaError_t pole_orbit_combine_scalar(double2* spec, const double2* part, int slices, const SymbolParams& sp,
+cudaError_t pole_orbit_combine_scalar(double2* spec, const void* part, int slices, const SymbolParams& sp,
                                       const OrbitParams& op, double2 phase, int adjoint, cudaStream_t s) {
   if (sp.spectral != 2) return cudaErrorInvalidValue;
   const size_t nk = (size_t)sp.nx * sp.ny;
-  pole_orbit_combine_scalar_kernel<<<(unsigned)((nk + 255) / 256), 256, 0, s>>>(spec, part, slices, sp.nx, sp.ny,
-                                                                                op, phase, adjoint);
+  pole_orbit_combine_scalar_kernel<<<(unsigned)((nk + 255) / 256), 256, 0, s>>>(
+      spec, static_cast<const double2*>(part), slices, sp.nx, sp.ny, op, phase, adjoint);
   return cudaGetLastError();
 }
 
-cudaError_t pole_orbit_combine_df(void* spec_df, const double2* part, int slices, void* fin, const SymbolParams& sp,
-                                  const float4* half_x_df, const float4* half_y_df, const OrbitParams& op,
-                                  const FusedScalars& fs, int row_len, cudaStream_t s) {
+cudaError_t pole_orbit_combine_df(void* spec_df, const void* fin, const SymbolParams& sp, const float4* half_x_df,
+                                  const float4* half_y_df, const OrbitParams& op, const FusedScalars& fs, int row_len,
+                                  cudaStream_t s) {
   if (fs.R0im != 0.0 || sp.spectral) return cudaErrorInvalidValue;  // real c0, s2 and the C-grid only
-  const double2 R0 = make_double2(fs.R0re, 0.0);
-  pole_orbit_finalize_kernel<true><<<(unsigned)((op.norb + 255) / 256), 256, 0, s>>>(part, slices, sp, op, R0, fin);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
   SymbolDF sd;
   sd.g = df_split_host(sp.g);
   sd.H = df_split_host(sp.H);
