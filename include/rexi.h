@@ -452,9 +452,10 @@ rexi_status rexi_batch_autotune(rexi_batch_t batch, const void* in_dev, void* ou
                                 int32_t* orbits_per_thread, double* best_ms);
 
 /* Current configuration and counters (each nullable): CTA size, orbits per
- * thread, persistent CTAs launched, work items, sum over instances of
- * wavenumber orbits x scalar terms (the pole-sum evaluations of one step),
- * kernels launched so far. */
+ * thread, persistent CTAs launched, work items (of the persistent kernel, and
+ * cells of the instances whose pole sum is expanded locally), sum over
+ * instances of wavenumber orbits x scalar terms (the evaluations that summing
+ * every orbit directly takes), kernels launched so far. */
 rexi_status rexi_batch_info(rexi_batch_t batch, int32_t* threads, int32_t* orbits_per_thread, int32_t* ctas,
                             int32_t* n_items, int64_t* terms_orbits, int64_t* launches);
 

@@ -751,7 +751,7 @@ rexi_status fourier_step(rexi_plan_s* p, const void* in, void* out, double dt, i
     const double x_lo = p->spectral == 2 ? tau * (p->lambda_min - p->sigma) : 0.0;
     const double x_hi = tau * (p->spectral == 2 ? -p->sigma : p->rho_natural);
     CellGeom cg;
-    const bool cells = cell_geometry(p->form, op.norb, fs.nterms, tb, te, h, q, x_lo, x_hi, G, &cg) &&
+    const bool cells = cell_geometry(p->form, op.norb, fs.nterms, tb, te, h, q, x_lo, x_hi, G, 0, &cg) &&
                        cell_scratch_values(cg) <= (size_t)L.slice_cap * op.norb;
     const void* raw = fin;  // kOrbitRaw: R+ of every orbit, as raw_slices partial sums
     int raw_slices = 1;

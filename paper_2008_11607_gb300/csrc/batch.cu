@@ -3,7 +3,9 @@
 //
 // The pole sum depends on a wavenumber only through omega(k), so it is
 // evaluated once per orbit of omega's symmetries (k -> -k per axis, and
-// kx <-> ky on square grids; see OrbitParams).  Work is split into items of
+// kx <-> ky on square grids; see OrbitParams).  Instances with enough orbits
+// and terms take the cells of pole_cells.cuh, one launch per level over all of
+// them; for the others the work is split into items of
 // `threads * orbits_per_thread` orbits of one instance; an item costs
 // (orbits x scalar terms).  Items are sorted by cost, largest first, and one
 // persistent kernel (a few CTAs per SM) pulls them from an atomic counter, so
@@ -80,6 +82,14 @@ struct rexi_batch_s {
   int* d_blk = nullptr;          // first combine block of each instance (n + 1 entries)
   int combine_blocks = 0;
   long long total_orbits = 0;
+  // instances whose pole sum takes the cells (cell_geometry): entry of
+  // cells.inst, or -1 for the persistent kernel's work items
+  std::vector<int> cell_of;
+  std::vector<rexi::CellGeom> cell_geom;  // per entry
+  rexi::CellBatch cells;
+  char* d_cells = nullptr;       // CellInst entries and the three lists
+  double* d_cell_tab = nullptr;  // cell_tables_host
+  long long cell_scratch = 0;    // double2 values
   std::vector<rexi::InstDesc> h_desc;
   long long total_terms_orbits = 0;
   // launch configuration of the persistent kernel
@@ -103,7 +113,7 @@ namespace {
 template <int FORM, int PPT>
 __global__ void batch_pole_kernel(OrbitScalars* orb, const InstDesc* __restrict__ desc,
                                   const WorkItem* __restrict__ items, int n_items, unsigned* counter,
-                                  const void* __restrict__ tables, double g, double f, double H) {
+                                  const void* __restrict__ tables, double g, double f, double H, int df) {
   __shared__ float4 st[kChunk * 3];  // 48 bytes per term, both forms
   __shared__ int s_item;
   __shared__ InstDesc D;
@@ -175,7 +185,10 @@ __global__ void batch_pole_kernel(OrbitScalars* orb, const InstDesc* __restrict_
       const double2 Rp = FORM == REXI_FORM_FP64
                              ? make_double2(ar[u], ai[u])
                              : make_double2((double)arh[u] + (double)arl[u], (double)aih[u] + (double)ail[u]);
-      orb[D.orb_off + o[u]] = orbit_scalars(om[u], make_double2(D.R0re, D.R0im), Rp);
+      if (FORM == REXI_FORM_MIXED && df && D.half_ok)
+        orbit_store<kOrbitDf>(orb + D.orb_off, o[u], om[u], make_double2(D.R0re, D.R0im), Rp);
+      else
+        orbit_store<kOrbitFp64>(orb + D.orb_off, o[u], om[u], make_double2(D.R0re, D.R0im), Rp);
     }
   }
 }
@@ -217,11 +230,14 @@ __global__ void __launch_bounds__(256) batch_combine_kernel(double2* spec, const
   op.sym = D.sym;
   op.norb = D.norb;
   const int ky = k / row_len, kx = k - ky * row_len;
-  OrbitScalars o = orb[D.orb_off + orbit_of(op, D.nx, D.ny, kx, ky)];
+  const int at = orbit_of(op, D.nx, D.ny, kx, ky);
+  OrbitScalars o;
+  if (!(half && df)) o = orb[D.orb_off + at];
   if (!half) {
     combine_scaled(spec + D.spec_off, (size_t)k, (size_t)nk, symbol_entries(sp, kx, ky, adjoint != 0),
                    make_double2(D.R0re, D.R0im), o, adjoint != 0);
   } else if (df) {
+    const OrbitScalarsDF od = reinterpret_cast<const OrbitScalarsDF*>(orb + D.orb_off)[at];
     SymbolDF sd;
     sd.g = g_df;
     sd.H = H_df;
@@ -231,7 +247,7 @@ __global__ void __launch_bounds__(256) batch_combine_kernel(double2* spec, const
     sd.half_x = D.halfdf_x;
     sd.half_y = D.halfdf_y;
     combine_df_at(reinterpret_cast<float4*>(spec + D.half_off), (size_t)k, (size_t)nk, kx, ky, sd,
-                  df_from_double(D.R0re), df_from_double(o.s1), df_from_double(o.s2re), adjoint != 0);
+                  df_from_double(D.R0re), od.s1, od.s2, adjoint != 0);
   } else {
     o.s2im = 0.0;
     combine_scaled(spec + D.half_off, (size_t)k, (size_t)nk, symbol_entries(sp, kx, ky, adjoint != 0),
@@ -240,7 +256,8 @@ __global__ void __launch_bounds__(256) batch_combine_kernel(double2* spec, const
 }
 
 template <int FORM, int PPT>
-cudaError_t launch_persistent(rexi_batch_s* b, OrbitScalars* orb, unsigned* counter, int threads, cudaStream_t s) {
+cudaError_t launch_persistent(rexi_batch_s* b, OrbitScalars* orb, unsigned* counter, int threads, int df,
+                              cudaStream_t s) {
   auto kern = batch_pole_kernel<FORM, PPT>;
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, 0);
@@ -250,16 +267,17 @@ cudaError_t launch_persistent(rexi_batch_s* b, OrbitScalars* orb, unsigned* coun
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int ctas = std::max(1, std::min(per_sm * sms, b->n_items));
   b->ctas = ctas;
-  kern<<<ctas, threads, 0, s>>>(orb, b->d_desc, b->d_items, b->n_items, counter, b->d_tables, b->g, b->f, b->H);
+  kern<<<ctas, threads, 0, s>>>(orb, b->d_desc, b->d_items, b->n_items, counter, b->d_tables, b->g, b->f, b->H,
+                                 df);
   return cudaGetLastError();
 }
 
-cudaError_t launch_pole(rexi_batch_s* b, OrbitScalars* orb, unsigned* counter, cudaStream_t s) {
+cudaError_t launch_pole(rexi_batch_s* b, OrbitScalars* orb, unsigned* counter, int df, cudaStream_t s) {
   if (b->form == REXI_FORM_FP64)
-    return b->ppt == 2 ? launch_persistent<REXI_FORM_FP64, 2>(b, orb, counter, b->threads, s)
-                       : launch_persistent<REXI_FORM_FP64, 1>(b, orb, counter, b->threads, s);
-  return b->ppt == 2 ? launch_persistent<REXI_FORM_MIXED, 2>(b, orb, counter, b->threads, s)
-                     : launch_persistent<REXI_FORM_MIXED, 1>(b, orb, counter, b->threads, s);
+    return b->ppt == 2 ? launch_persistent<REXI_FORM_FP64, 2>(b, orb, counter, b->threads, df, s)
+                       : launch_persistent<REXI_FORM_FP64, 1>(b, orb, counter, b->threads, df, s);
+  return b->ppt == 2 ? launch_persistent<REXI_FORM_MIXED, 2>(b, orb, counter, b->threads, df, s)
+                     : launch_persistent<REXI_FORM_MIXED, 1>(b, orb, counter, b->threads, df, s);
 }
 
 cudaError_t launch_combine(rexi_batch_s* b, double2* spec, const OrbitScalars* orb, int real_input, cudaStream_t s) {
@@ -271,7 +289,7 @@ cudaError_t launch_combine(rexi_batch_s* b, double2* spec, const OrbitScalars* o
 
 size_t al256(size_t v) { return (v + 255) / 256 * 256; }
 
-// Workspace: [counter (256 B)][packed spectrum][per-orbit R+ of every instance]
+// Workspace: [counter (256 B)][packed spectrum][per-orbit combine scalars of every instance][cells]
 size_t batch_spec_bytes(const rexi_batch_s* b) { return al256((size_t)b->offsets[b->n] * sizeof(double2)); }
 // The orbit region also serves the per-instance mode, one instance at a
 // time: its term slices' partial sums, then its combine scalars.
@@ -283,7 +301,10 @@ size_t batch_orb_bytes(const rexi_batch_s* b) {
   for (const auto& D : b->h_desc) m = std::max(m, per_instance_part_bytes(D) + orbit_scalars_bytes(D.norb));
   return m;
 }
-size_t batch_ws_bytes(const rexi_batch_s* b) { return 256 + batch_spec_bytes(b) + al256(batch_orb_bytes(b)); }
+size_t batch_cells_off(const rexi_batch_s* b) { return 256 + batch_spec_bytes(b) + al256(batch_orb_bytes(b)); }
+size_t batch_ws_bytes(const rexi_batch_s* b) {
+  return batch_cells_off(b) + al256((size_t)b->cell_scratch * sizeof(double2));
+}
 
 // (Re)build the work items for the current item size, largest cost first.
 cudaError_t build_items(rexi_batch_s* b) {
@@ -295,12 +316,16 @@ cudaError_t build_items(rexi_batch_s* b) {
   };
   std::vector<Cost> v;
   for (int i = 0; i < b->n; ++i) {
+    if (b->cell_of[i] >= 0) continue;
     const int no = b->h_desc[i].norb;
     for (int p = 0; p < no; p += item_orbits) {
       const long long orbits = std::min(item_orbits, no - p);
       v.push_back({orbits * (long long)b->h_desc[i].nterms, {i, p}});
     }
   }
+  b->item_orbits = item_orbits;
+  b->n_items = (int)v.size();
+  if (v.empty()) return cudaSuccess;  // every instance takes the cells
   std::stable_sort(v.begin(), v.end(), [](const Cost& a, const Cost& c) { return a.cost > c.cost; });
   std::vector<WorkItem> items(v.size());
   for (size_t k = 0; k < v.size(); ++k) items[k] = v[k].w;
@@ -309,9 +334,92 @@ cudaError_t build_items(rexi_batch_s* b) {
   cudaError_t e = cudaMalloc(&b->d_items, items.size() * sizeof(WorkItem));
   if (e != cudaSuccess) return e;
   e = cudaMemcpy(b->d_items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice);
-  b->n_items = (int)items.size();
-  b->item_orbits = item_orbits;
   return e;
+}
+
+SymbolParams symbol_of(const rexi_batch_s* b, const InstDesc& D) {
+  SymbolParams sp;
+  sp.nx = D.nx;
+  sp.ny = D.ny;
+  sp.inv_dx = D.inv_dx;
+  sp.inv_dy = D.inv_dy;
+  sp.g = b->g;
+  sp.f = b->f;
+  sp.H = b->H;
+  sp.half_x = D.half_x;
+  sp.half_y = D.half_y;
+  return sp;
+}
+OrbitParams orbits_of(const InstDesc& D) {
+  OrbitParams op;
+  op.ax = D.ax;
+  op.ay = D.ay;
+  op.sym = D.sym;
+  op.norb = D.norb;
+  return op;
+}
+
+// Uploads the coefficient tables, decides per instance between the cells and
+// the persistent kernel (the rule of the single-instance step), and uploads
+// the cells' descriptors and block lists.
+bool build_cells(rexi_batch_s* b, const char* tab, size_t tab_bytes) {
+  if (cudaMalloc(&b->d_tables, tab_bytes) != cudaSuccess ||
+      cudaMemcpy(b->d_tables, tab, tab_bytes, cudaMemcpyHostToDevice) != cudaSuccess)
+    return false;
+  std::vector<CellInst> inst;
+  std::vector<int2> far, cell, orbit;
+  b->cell_of.assign(b->n, -1);
+  for (int i = 0; i < b->n; ++i) {
+    const InstDesc& D = b->h_desc[i];
+    CellInst I{};
+    if (!cell_geometry(b->form, D.norb, D.nterms, 0, (D.nterms + 1) / 2, b->h, D.q, 0.0, D.tau * b->rho[i],
+                       b->form == REXI_FORM_MIXED ? D.grid : 0.0, 1, &I.g) ||
+        cell_scratch_values(I.g) > (size_t)orbit_slice_cap(D.norb) * D.norb || far.size() + I.g.ncoarse > 65535)
+      continue;
+    const int at = (int)inst.size();
+    b->cell_of[i] = at;
+    I.sp = symbol_of(b, D);
+    I.op = orbits_of(D);
+    I.R0 = make_double2(D.R0re, D.R0im);
+    I.tau = D.tau;
+    I.table = static_cast<const char*>(b->d_tables) + D.table_off * 48;
+    I.scratch_off = b->cell_scratch;
+    I.orb_off = D.orb_off;
+    I.exact_hn = D.exact_hn;
+    I.half_ok = D.half_ok;
+    b->cell_scratch += (long long)cell_scratch_values(I.g);
+    if (I.g.two_level)
+      for (int c = 0; c < I.g.ncoarse; ++c) far.push_back(make_int2(at, c));
+    for (int c = 0; c < I.g.ncell; ++c) cell.push_back(make_int2(at, c));
+    for (int o = 0; o < D.norb; o += 256) orbit.push_back(make_int2(at, o));
+    inst.push_back(I);
+    b->cell_geom.push_back(I.g);
+  }
+  if (inst.empty()) return true;
+  // blocks with the most terms first, so that none of the long ones starts last
+  auto heavier = [&](const int2& p, const int2& q) { return inst[p.x].g.nterms > inst[q.x].g.nterms; };
+  std::stable_sort(far.begin(), far.end(), heavier);
+  const size_t bi = al256(inst.size() * sizeof(CellInst)), bf = al256(far.size() * sizeof(int2)),
+               bc = al256(cell.size() * sizeof(int2)), bo = orbit.size() * sizeof(int2);
+  const std::vector<double>& ct = cell_tables_host();
+  if (cudaMalloc(&b->d_cells, bi + bf + bc + bo) != cudaSuccess ||
+      cudaMalloc(&b->d_cell_tab, ct.size() * sizeof(double)) != cudaSuccess)
+    return false;
+  auto put = [&](size_t off, const void* src, size_t bytes) {
+    return bytes == 0 || cudaMemcpy(b->d_cells + off, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
+  };
+  if (!put(0, inst.data(), inst.size() * sizeof(CellInst)) || !put(bi, far.data(), far.size() * sizeof(int2)) ||
+      !put(bi + bf, cell.data(), cell.size() * sizeof(int2)) || !put(bi + bf + bc, orbit.data(), bo) ||
+      cudaMemcpy(b->d_cell_tab, ct.data(), ct.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
+    return false;
+  b->cells.inst = reinterpret_cast<const CellInst*>(b->d_cells);
+  b->cells.far = reinterpret_cast<const int2*>(b->d_cells + bi);
+  b->cells.cell = reinterpret_cast<const int2*>(b->d_cells + bi + bf);
+  b->cells.orbit = reinterpret_cast<const int2*>(b->d_cells + bi + bf + bc);
+  b->cells.n_far = (int)far.size();
+  b->cells.n_cell = (int)cell.size();
+  b->cells.n_orbit = (int)orbit.size();
+  return true;
 }
 
 // FP64 transforms for the FP64 form, double-float ones for the mixed form.
@@ -338,7 +446,10 @@ cudaError_t enqueue_persistent(rexi_batch_s* b, const double2* in, double2* out,
       e = fft_any(b, in + G.first_off, spec + G.first_off, nf, G.fx, G.fy, -1, 1.0, real_input, 0, s);
   }
   if (e != cudaSuccess) return e;
-  e = launch_pole(b, orb, counter, s);
+  if (b->n_items > 0) e = launch_pole(b, orb, counter, real_input && df, s);
+  if (e == cudaSuccess && b->cells.n_cell > 0)
+    e = pole_cells_batch(b->form, b->cells, cell_tables_at(b->d_cell_tab),
+                         reinterpret_cast<double2*>(ws + batch_cells_off(b)), orb, real_input && df, s);
   if (e == cudaSuccess) e = launch_combine(b, spec, orb, real_input, s);
   for (auto& G : b->groups) {
     if (e != cudaSuccess) return e;
@@ -381,6 +492,8 @@ void rexi_batch_destroy(rexi_batch_t b) {
   cudaFree(b->d_desc);
   cudaFree(b->d_items);
   cudaFree(b->d_blk);
+  cudaFree(b->d_cells);
+  cudaFree(b->d_cell_tab);
   delete b;
 }
 
@@ -592,15 +705,15 @@ rexi_status rexi_batch_create(rexi_batch_t* out, int32_t n, const int32_t* nx, c
       D.halfdf_y = b->axis_halfdf[G.ny];
     }
   }
+  if (!build_cells(b, reinterpret_cast<const char*>(tab.data()), tab.size() * sizeof(float)))
+    return bail(REXI_ENOMEM, "rexi_batch_create: device allocation failed");
   std::vector<int> blk(n + 1, 0);
   for (int i = 0; i < n; ++i) blk[i + 1] = blk[i] + (b->nx[i] * b->ny[i] + 255) / 256;
   b->combine_blocks = blk[n];
-  if (cudaMalloc(&b->d_tables, tab.size() * sizeof(float)) != cudaSuccess ||
-      cudaMalloc(&b->d_desc, n * sizeof(InstDesc)) != cudaSuccess ||
+  if (cudaMalloc(&b->d_desc, n * sizeof(InstDesc)) != cudaSuccess ||
       cudaMalloc(&b->d_blk, (n + 1) * sizeof(int)) != cudaSuccess)
     return bail(REXI_ENOMEM, "rexi_batch_create: device allocation failed");
   cudaMemcpy(b->d_blk, blk.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice);
-  cudaMemcpy(b->d_tables, tab.data(), tab.size() * sizeof(float), cudaMemcpyHostToDevice);
   cudaMemcpy(b->d_desc, b->h_desc.data(), n * sizeof(InstDesc), cudaMemcpyHostToDevice);
   if (build_items(b) != cudaSuccess) return bail(REXI_ENOMEM, "rexi_batch_create: work list allocation failed");
   if (cudaStreamCreateWithFlags(&b->own, cudaStreamNonBlocking) != cudaSuccess ||
@@ -667,26 +780,28 @@ rexi_status rexi_batch_step(rexi_batch_t b, const void* in, void* out, int32_t r
       } else {
         e = fft_any(b, in2 + D.spec_off, sp_i, 3, fx, fy, -1, 1.0, real_input, 0, s);
       }
-      SymbolParams sp;
-      sp.nx = D.nx; sp.ny = D.ny; sp.inv_dx = D.inv_dx; sp.inv_dy = D.inv_dy;
-      sp.g = b->g; sp.f = b->f; sp.H = b->H; sp.half_x = D.half_x; sp.half_y = D.half_y;
+      const SymbolParams sp = symbol_of(b, D);
       FusedScalars fs;
       fs.tau = D.tau; fs.q = D.q; fs.R0re = D.R0re; fs.R0im = half ? 0.0 : D.R0im; fs.nterms = D.nterms;
       fs.adjoint = 0;
       fs.exact_hn = D.exact_hn;  // the instance's table: whether every h n lies on its split grid
       const float* tab = static_cast<const float*>(b->d_tables) + D.table_off * 12;
-      // the single-instance kernels, term slices as rexi_step chooses them
-      OrbitParams op;
-      op.ax = D.ax; op.ay = D.ay; op.sym = D.sym; op.norb = D.norb;
-      const int slices = pole_orbit_slices(b->form, op.norb, D.nterms, orbit_slice_cap(op.norb));
+      // the single-instance kernels: cells or term slices as rexi_step chooses them
+      const OrbitParams op = orbits_of(D);
       double2* part = reinterpret_cast<double2*>(orb);
-      if (e == cudaSuccess)
-        e = b->form == REXI_FORM_FP64
-                ? pole_orbits_fp64(part, slices, sp, op, reinterpret_cast<const double*>(tab), fs, s)
-                : pole_orbits_mixed(part, slices, sp, op, tab, fs, D.grid, s);
       void* fin = orb + per_instance_part_bytes(D);
-      if (e == cudaSuccess)
-        e = pole_orbit_finalize(part, slices, sp, op, fs, half && df ? kOrbitDf : kOrbitFp64, fin, s);
+      const OrbitOut kind = half && df ? kOrbitDf : kOrbitFp64;
+      if (e == cudaSuccess && b->cell_of[i] >= 0) {
+        e = pole_cells(b->form, b->cell_geom[b->cell_of[i]], cell_tables_at(b->d_cell_tab), tab, part, sp, op, fs,
+                       kind, fin, s);
+      } else {
+        const int slices = pole_orbit_slices(b->form, op.norb, D.nterms, orbit_slice_cap(op.norb));
+        if (e == cudaSuccess)
+          e = b->form == REXI_FORM_FP64
+                  ? pole_orbits_fp64(part, slices, sp, op, reinterpret_cast<const double*>(tab), fs, s)
+                  : pole_orbits_mixed(part, slices, sp, op, tab, fs, D.grid, s);
+        if (e == cudaSuccess) e = pole_orbit_finalize(part, slices, sp, op, fs, kind, fin, s);
+      }
       const double scale = 1.0 / ((double)D.nx * D.ny);
       if (e == cudaSuccess) {
         if (half && df)
@@ -730,7 +845,8 @@ rexi_status rexi_batch_step(rexi_batch_t b, const void* in, void* out, int32_t r
     if (e == cudaSuccess) e = cudaGraphLaunch(b->exec, b->own);
     if (e == cudaSuccess) e = cudaEventRecord(b->ev_out, b->own);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, b->ev_out, 0);
-    b->launches += 2 + 4 * (int64_t)b->groups.size();
+    b->launches += 1 + (b->n_items > 0 ? 1 : 0) + (b->cells.n_cell > 0 ? 2 + (b->cells.n_far > 0 ? 1 : 0) : 0) +
+                   4 * (int64_t)b->groups.size();
   } else {
     set_last_error("rexi_batch_step: unknown mode");
     return REXI_EINVAL;
@@ -795,7 +911,7 @@ rexi_status rexi_batch_info(rexi_batch_t b, int32_t* threads, int32_t* ppt, int3
   if (threads) *threads = b->threads;
   if (ppt) *ppt = b->ppt;
   if (ctas) *ctas = b->ctas;
-  if (n_items) *n_items = b->n_items;
+  if (n_items) *n_items = b->n_items + b->cells.n_cell;
   if (terms_orbits) *terms_orbits = b->total_terms_orbits;
   if (launches) *launches = b->launches;
   return REXI_OK;

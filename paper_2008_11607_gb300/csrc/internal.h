@@ -153,14 +153,37 @@ struct CellTables {  // device tables, the same for every plan (cell_tables_host
 };
 const std::vector<double>& cell_tables_host();
 CellTables cell_tables_at(const double* dev);
-// The cells for x in [x_lo, x_hi], or false where summing every orbit directly costs less.
+// The cells for x in [x_lo, x_hi], or false where summing every orbit directly
+// costs less (shared_launches: the launches serve many instances).
 bool cell_geometry(int form, int norb, int nterms, int tb, int te, double h, double q, double x_lo, double x_hi,
-                   double grid, CellGeom* g);
+                   double grid, int shared_launches, CellGeom* g);
 size_t cell_scratch_values(const CellGeom& g);  // double2 values of scratch
 // fin of every orbit, as pole_orbits_* and pole_orbit_finalize leave it.
 cudaError_t pole_cells(int form, const CellGeom& g, const CellTables& T, const void* table, double2* scratch,
                        const SymbolParams& sp, const OrbitParams& op, const FusedScalars& fs, OrbitOut kind,
                        void* fin, cudaStream_t s);
+// The same for the instances of a batch that take the cells: device lists of
+// (entry of inst, coarse cell / cell / first orbit) per block; orb: 32 bytes
+// per orbit of the batch, the FP64 combine scalars, or with df (real input in
+// the mixed form) OrbitScalarsDF from the start of an instance's range where
+// its real transforms are available (half_ok).
+struct CellInst {
+  CellGeom g;
+  SymbolParams sp;
+  OrbitParams op;
+  double2 R0;
+  double tau;
+  const void* table;
+  long long scratch_off, orb_off;  // double2 values; OrbitScalars entries
+  int exact_hn, half_ok;
+};
+struct CellBatch {
+  const CellInst* inst = nullptr;
+  const int2 *far = nullptr, *cell = nullptr, *orbit = nullptr;
+  int n_far = 0, n_cell = 0, n_orbit = 0;  // n_far <= 65535 (a grid's y extent)
+};
+cudaError_t pole_cells_batch(int form, const CellBatch& b, const CellTables& T, double2* scratch, void* orb, int df,
+                             cudaStream_t s);
 
 // spec <- r(tau B) spec at every wavenumber from the orbits' scalars.
 // row_len: nx (full spectrum, rows of nx values) or nx/2 + 1 (half spectrum

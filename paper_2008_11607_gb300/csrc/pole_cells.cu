@@ -2,14 +2,16 @@
 //
 // What bounds it, and the split.  Direct sums cost orbits x terms evaluations
 // of 62 FP32 operations (mixed) or 9 FP64 instructions; the cells cost nodes
-// x near terms + coarse nodes x far terms.  The far kernel gives a warp to
-// each coarse node (24 per 32 cells), the cell kernel 16 lanes to each node,
-// so that both have warps for every SM and short chains; what is left is one
-// polynomial per orbit in FP64, about 45 dependent operations, and the orbit's
-// omega.  Measured (GB300): 2048^2, tau rho = 1000, 525,825 orbits x 4067
-// terms, direct 4286 us (mixed) and 32,902 us (FP64), cells 166 us and 225 us;
-// 375 x 500, tau rho = 150, FP64, 47,188 orbits x 667 terms, 521 us against
-// 40 us.  Error against 64 bits as the direct sums' or smaller (shorter sums).
+// x near terms + coarse nodes x far terms.  The far kernel gives a block to
+// each coarse node (24 per 32 cells), the cell kernel 8 or 32 lanes to each
+// node, so that both have warps for every SM and short chains; what is left is
+// one polynomial per orbit and the orbit's omega, where every FP64 instruction
+// counts (one takes the time of about 60 FP32 ones).  Measured (GB300): 2048^2, tau rho = 1000, 525,825 orbits x 4067
+// terms, direct 4286 us (mixed) and 32,902 us (FP64), cells 75 us and 185 us
+// (166 and 225 us with 16 FP64 lanes per node and the library's root and
+// division per orbit); the serving mix of 96 instances, mixed, 3088 us in the
+// persistent kernel, 356 us with cells; 375 x 500, tau rho = 150, FP64, 47,188
+// orbits x 667 terms, 521 us against 36 us.  Error against 64 bits as the direct sums' or smaller (shorter sums).
 #include <math.h>
 
 #include <algorithm>
@@ -20,34 +22,99 @@ namespace rexi {
 
 namespace {
 
-constexpr int kFarWarps = 4;
-static_assert(kCellPC % kFarWarps == 0, "a block's warps belong to one coarse cell");
-static_assert(kCellP == 16, "cell_poly's lanes");
+static_assert(kCellP == 16 && kCellPC % 2 == 0, "cell_poly's second part");
+// Lanes per node: 8, or 32 where fewer cells than this leave a multiprocessor
+// with less than four blocks, whose chains of terms then set the time (360 x
+// 250, tau rho = 120, 121 cells x 547 terms).
+constexpr int kWideCells = 600;
 
 template <int FORM>
-__global__ void __launch_bounds__(kFarWarps * 32) cell_far_kernel(CellGeom g, CellTables T,
-                                                                  const void* __restrict__ table, double2* far) {
-  cell_far_node<FORM>(g, table, T, blockIdx.y, blockIdx.x * kFarWarps + (threadIdx.x >> 5), far);
+__global__ void __launch_bounds__(kFarThreads) cell_far_kernel(CellGeom g, CellTables T,
+                                                               const void* __restrict__ table, double2* far) {
+  __shared__ double2 red[kFarThreads / 32];
+  cell_far_node<FORM>(g, table, T, blockIdx.y, blockIdx.x, far, red);
 }
 
-template <int FORM>
-__global__ void __launch_bounds__(kCellP * 16) cell_poly_kernel(CellGeom g, CellTables T,
-                                                                const void* __restrict__ table,
-                                                                const double2* __restrict__ far, double2* poly) {
-  __shared__ double2 sh[2 * kCellP];
-  cell_poly<FORM>(g, table, T, blockIdx.x, far, poly, sh);
+template <int FORM, bool DF, int LANES>
+__global__ void __launch_bounds__(LANES* kCellP) cell_poly_kernel(CellGeom g, CellTables T,
+                                                                  const void* __restrict__ table,
+                                                                  const double2* __restrict__ far, void* poly) {
+  __shared__ CellShared<FORM> sh;
+  cell_poly<FORM, DF, LANES>(g, table, T, blockIdx.x, far, poly, sh);
+}
+template <int LANES>
+void launch_poly(int f, bool df, const CellGeom& g, const CellTables& T, const void* table, const double2* far,
+                 void* poly, cudaStream_t s) {
+  auto k = f == 0   ? (df ? cell_poly_kernel<0, true, LANES> : cell_poly_kernel<0, false, LANES>)
+           : f == 1 ? (df ? cell_poly_kernel<1, true, LANES> : cell_poly_kernel<1, false, LANES>)
+                    : (df ? cell_poly_kernel<2, true, LANES> : cell_poly_kernel<2, false, LANES>);
+  k<<<(unsigned)g.ncell, LANES * kCellP, 0, s>>>(g, T, table, far, poly);
 }
 
-template <int KIND>
-__global__ void __launch_bounds__(256) cell_orbits_kernel(CellGeom g, const double2* __restrict__ poly,
-                                                          SymbolParams sp, OrbitParams op, double tau, double2 R0,
+template <int KIND, bool CGRID>
+__global__ void __launch_bounds__(256) cell_orbits_kernel(CellGeom g, const void* __restrict__ poly, SymbolParams sp,
+                                                          OrbitParams op, double tau, double2 R0,
                                                           void* __restrict__ fin) {
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= op.norb) return;
-  int a, b;
-  orbit_rep(op, o, a, b);
-  const double omega = symbol_at(sp, a, b).omega;
-  orbit_store<KIND>(fin, o, omega, R0, cell_eval(g, poly, tau * omega));
+  if (o < op.norb) cell_orbit<KIND, CGRID>(g, poly, sp, op, tau, R0, o, fin);
+}
+
+// The same over the instances of a batch: a block looks its (instance, cell)
+// up in a flat list.
+template <bool MIXED>
+__global__ void __launch_bounds__(kFarThreads) batch_far_kernel(const CellInst* __restrict__ inst,
+                                                                const int2* __restrict__ list, CellTables T,
+                                                                double2* scratch) {
+  __shared__ double2 red[kFarThreads / 32];
+  const int2 e = list[blockIdx.y];
+  const CellInst& I = inst[e.x];
+  double2* far = scratch + I.scratch_off + (size_t)I.g.ncell * kCellP;
+  if (!MIXED)
+    cell_far_node<0>(I.g, I.table, T, e.y, blockIdx.x, far, red);
+  else if (I.exact_hn)
+    cell_far_node<1>(I.g, I.table, T, e.y, blockIdx.x, far, red);
+  else
+    cell_far_node<2>(I.g, I.table, T, e.y, blockIdx.x, far, red);
+}
+template <bool MIXED>
+__global__ void __launch_bounds__(8 * kCellP) batch_poly_kernel(const CellInst* __restrict__ inst,
+                                                                const int2* __restrict__ list, CellTables T,
+                                                                double2* scratch, int df) {
+  const int2 e = list[blockIdx.x];
+  const CellInst& I = inst[e.x];
+  double2* poly = scratch + I.scratch_off;
+  const double2* far = poly + (size_t)I.g.ncell * kCellP;
+  const bool pairs = df && I.half_ok;
+  if constexpr (!MIXED) {
+    __shared__ CellShared<0> sh;
+    cell_poly<0, false, 8>(I.g, I.table, T, e.y, far, poly, sh);
+  } else if (I.exact_hn) {
+    __shared__ CellShared<1> sh;
+    if (pairs)
+      cell_poly<1, true, 8>(I.g, I.table, T, e.y, far, poly, sh);
+    else
+      cell_poly<1, false, 8>(I.g, I.table, T, e.y, far, poly, sh);
+  } else {
+    __shared__ CellShared<2> sh;
+    if (pairs)
+      cell_poly<2, true, 8>(I.g, I.table, T, e.y, far, poly, sh);
+    else
+      cell_poly<2, false, 8>(I.g, I.table, T, e.y, far, poly, sh);
+  }
+}
+__global__ void __launch_bounds__(256) batch_orbits_kernel(const CellInst* __restrict__ inst,
+                                                           const int2* __restrict__ list,
+                                                           const double2* __restrict__ scratch,
+                                                           OrbitScalars* __restrict__ orb, int df) {
+  const int2 e = list[blockIdx.x];
+  const CellInst& I = inst[e.x];
+  const int o = e.y + threadIdx.x;
+  if (o >= I.op.norb) return;
+  void* fin = orb + I.orb_off;
+  if (df && I.half_ok)
+    cell_orbit<kOrbitDf, true>(I.g, scratch + I.scratch_off, I.sp, I.op, I.tau, I.R0, o, fin);
+  else
+    cell_orbit<kOrbitFp64, true>(I.g, scratch + I.scratch_off, I.sp, I.op, I.tau, I.R0, o, fin);
 }
 
 typedef long double ld;
@@ -147,7 +214,7 @@ CellTables cell_tables_at(const double* dev) {
 }
 
 bool cell_geometry(int form, int norb, int nterms, int tb, int te, double h, double q, double x_lo, double x_hi,
-                   double grid, CellGeom* g) {
+                   double grid, int shared_launches, CellGeom* g) {
   if (nterms < 1 || !(q > 0.0) || !(x_hi >= x_lo)) return false;
   const double a = sqrt(q);
   g->c = ldexp(1.0, (int)floor(log2(a / 5.13)));
@@ -169,13 +236,14 @@ bool cell_geometry(int form, int norb, int nterms, int tb, int te, double h, dou
   g->k0 = (int)k0;
   g->ncell = (int)(k1 - k0) + 1;
   g->ncoarse = (g->ncell + kCellK - 1) / kCellK;
-  // Costs in term evaluations: a launch is worth about 4 us of them, a
-  // polynomial 32 FP64 instructions.  The cells win as soon as the orbits
+  // Costs in term evaluations: a launch is worth about 4 us of them
+  // (shared by the instances of a batch).  The cells win as soon as the orbits
   // outnumber the nodes by enough to pay for the extra launches: 360 x 250,
-  // tau rho = 120, mixed (22,806 orbits, 1936 nodes) 52 us direct, 30 us with
+  // tau rho = 120, mixed (22,806 orbits, 1936 nodes) 52 us direct, 22 us with
   // cells; 64^2, tau rho = 50 (561 orbits, 816 nodes) stays direct.
   const bool mixed = form == REXI_FORM_MIXED;
-  const double launch = mixed ? 2.0e6 : 2.7e5, poly = mixed ? 27.0 : 4.0;
+  const double launch = (mixed ? 2.0e6 : 2.7e5) * (shared_launches ? 0.02 : 1.0);
+  const double poly = mixed ? 12.0 : 6.0;  // an orbit's omega and polynomial
   const double near = std::min<double>(nterms, 5.0 * kCellK * g->c * g->inv_h);
   const double nodes = (double)g->ncell * kCellP;
   const double one = nodes * nterms;
@@ -196,18 +264,39 @@ cudaError_t pole_cells(int form, const CellGeom& g, const CellTables& T, const v
   const int f = form == REXI_FORM_MIXED ? (fs.exact_hn ? 1 : 2) : 0;
   cudaError_t e;
   if (g.two_level) {
-    const dim3 grid(kCellPC / kFarWarps, (unsigned)g.ncoarse);
     auto k = f == 0 ? cell_far_kernel<0> : f == 1 ? cell_far_kernel<1> : cell_far_kernel<2>;
-    k<<<grid, kFarWarps * 32, 0, s>>>(g, T, table, far);
+    k<<<dim3(kCellPC, (unsigned)g.ncoarse), kFarThreads, 0, s>>>(g, T, table, far);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  auto kp = f == 0 ? cell_poly_kernel<0> : f == 1 ? cell_poly_kernel<1> : cell_poly_kernel<2>;
-  kp<<<(unsigned)g.ncell, kCellP * 16, 0, s>>>(g, T, table, far, poly);
+  const bool df = kind == kOrbitDf;
+  if (g.ncell <= kWideCells)
+    launch_poly<32>(f, df, g, T, table, far, poly, s);
+  else
+    launch_poly<8>(f, df, g, T, table, far, poly, s);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  auto ko = kind == kOrbitFp64 ? cell_orbits_kernel<kOrbitFp64>
-            : kind == kOrbitDf ? cell_orbits_kernel<kOrbitDf>
-                               : cell_orbits_kernel<kOrbitRaw>;
+  const bool cgrid = sp.spectral == 0;
+  auto ko = kind == kOrbitDf     ? cell_orbits_kernel<kOrbitDf, true>
+            : kind == kOrbitRaw  ? cell_orbits_kernel<kOrbitRaw, false>
+            : cgrid              ? cell_orbits_kernel<kOrbitFp64, true>
+                                 : cell_orbits_kernel<kOrbitFp64, false>;
   ko<<<(unsigned)((op.norb + 255) / 256), 256, 0, s>>>(g, poly, sp, op, fs.tau, make_double2(fs.R0re, fs.R0im), fin);
+  return cudaGetLastError();
+}
+
+cudaError_t pole_cells_batch(int form, const CellBatch& b, const CellTables& T, double2* scratch, void* orb, int df,
+                             cudaStream_t s) {
+  const bool mixed = form == REXI_FORM_MIXED;
+  cudaError_t e;
+  if (b.n_far > 0) {
+    auto k = mixed ? batch_far_kernel<true> : batch_far_kernel<false>;
+    k<<<dim3(kCellPC, (unsigned)b.n_far), kFarThreads, 0, s>>>(b.inst, b.far, T, scratch);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  auto k = mixed ? batch_poly_kernel<true> : batch_poly_kernel<false>;
+  k<<<(unsigned)b.n_cell, 8 * kCellP, 0, s>>>(b.inst, b.cell, T, scratch, df);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  batch_orbits_kernel<<<(unsigned)b.n_orbit, 256, 0, s>>>(b.inst, b.orbit, scratch, static_cast<OrbitScalars*>(orb),
+                                                          df);
   return cudaGetLastError();
 }
 

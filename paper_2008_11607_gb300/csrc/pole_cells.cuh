@@ -28,10 +28,9 @@
 namespace rexi {
 
 // First index of the table's terms (n ascending, |n| in [tb, te)) with n >= v.
-__device__ __forceinline__ int cell_term_at(const CellGeom& g, double v) {
+__device__ __forceinline__ int cell_term_at(const CellGeom& g, float v) {
   // tb = 0: n = -(te - 1)..te - 1; tb > 0: the two runs -(te - 1)..-tb and tb..te - 1
-  const double n = fmin(fmax(ceil(v), -(double)g.te), (double)g.te);
-  const int ni = (int)n;
+  const int ni = (int)fminf(fmaxf(ceilf(v), -(float)g.te), (float)g.te);
   if (g.tb == 0) return min(max(ni + g.te - 1, 0), g.nterms);
   const int run = g.te - g.tb;
   if (ni <= -g.tb) return max(ni + g.te - 1, 0);
@@ -39,125 +38,272 @@ __device__ __forceinline__ int cell_term_at(const CellGeom& g, double v) {
   return min(run + ni - g.tb, g.nterms);
 }
 
-// Terms summed at the cells of coarse cell cc themselves: [lo, hi).
+// Terms summed at the cells of coarse cell cc themselves: [lo, hi).  FP32
+// (FP64 instructions are dear here): the far and the cell kernel call the same
+// function, so a boundary term that rounds either way is still in exactly one sum.
 __device__ __forceinline__ void cell_near(const CellGeom& g, int cc, int& lo, int& hi) {
   if (!g.two_level) {
     lo = 0;
     hi = g.nterms;
     return;
   }
-  const double C = kCellK * g.c, Xc = (double)(g.k0 + cc * kCellK) * g.w + C;
-  lo = cell_term_at(g, (-Xc - 2.5 * C) * g.inv_h);
-  hi = max(lo, cell_term_at(g, (-Xc + 2.5 * C) * g.inv_h));
+  const float C = kCellK * (float)g.c, Xc = (float)(g.k0 + cc * kCellK) * (float)g.w + C;
+  lo = cell_term_at(g, (-Xc - 2.5f * C) * (float)g.inv_h);
+  hi = max(lo, cell_term_at(g, (-Xc + 2.5f * C) * (float)g.inv_h));
 }
 
-// Sum of the table's terms first, first + stride, ... below `end` at x.
+// Partial sums of R+ in the form's arithmetic.
 template <int FORM>  // 0 FP64, 1 double-float with h n on the split grid, 2 double-float otherwise
-__device__ __forceinline__ void cell_terms(const CellGeom& g, const void* table, double x, int first, int end,
-                                           int stride, double& re, double& im) {
-  if (FORM == 0) {
+struct CellAcc {
+  float2 re = {0.f, 0.f}, im = {0.f, 0.f};
+};
+template <>
+struct CellAcc<0> {
+  double re = 0.0, im = 0.0;
+};
+__device__ __forceinline__ double cell_add(double a, double b) { return a + b; }
+__device__ __forceinline__ float2 cell_add(float2 a, float2 b) { return f_add(a.x, a.y, b.x, b.y); }
+__device__ __forceinline__ double cell_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ float2 cell_xor(float2 v, int o) {
+  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
+}
+__device__ __forceinline__ double cell_f64(double v) { return v; }
+__device__ __forceinline__ double cell_f64(float2 v) { return df_to_double(v); }
+
+// x as the form's terms take it: FP64, or X_hi on the split grid + X_lo + X_lo2.
+template <int FORM>
+struct CellX {
+  float h, l, l2;
+};
+template <>
+struct CellX<0> {
+  double x;
+};
+template <int FORM>
+__device__ __forceinline__ CellX<FORM> cell_x(const CellGeom& g, double x) {
+  if constexpr (FORM == 0) {
+    return {x};
+  } else {
+    const double xg = rint(x * g.inv_grid) * g.grid, r = x - xg;
+    const float l = (float)r;
+    return {(float)xg, l, (float)(r - (double)l)};
+  }
+}
+
+// acc += the table's terms first, first + stride, ... below `end` at X.
+template <int FORM>
+__device__ __forceinline__ void cell_terms(const CellGeom& g, const void* table, const CellX<FORM>& X, int first,
+                                           int end, int stride, CellAcc<FORM>& acc) {
+  if constexpr (FORM == 0) {
     const double2* tb = static_cast<const double2*>(table);
 #pragma unroll 2
-    for (int t = first; t < end; t += stride) fp64_term(tb + 3 * (size_t)t, x, g.q, re, im);
+    for (int t = first; t < end; t += stride) fp64_term(tb + 3 * (size_t)t, X.x, g.q, acc.re, acc.im);
   } else {
     const float4* tb = static_cast<const float4*>(table);
-    const double xg = rint(x * g.inv_grid) * g.grid;
-    const float Xh = (float)xg, Xl = (float)(x - xg), Xl2 = (float)((x - xg) - (double)Xl);
-    float arh = 0.f, arl = 0.f, aih = 0.f, ail = 0.f;
     int k = 0;
 #pragma unroll 2
     for (int t = first; t < end; t += stride) {
-      df_term<FORM == 1>(tb + 3 * (size_t)t, Xh, Xl, Xl2, g.q_hi, g.q_lo, arh, arl, aih, ail);
+      df_term<FORM == 1>(tb + 3 * (size_t)t, X.h, X.l, X.l2, g.q_hi, g.q_lo, acc.re.x, acc.re.y, acc.im.x, acc.im.y);
       if ((++k & (kRenorm - 1)) == 0) {
-        df_renorm(arh, arl);
-        df_renorm(aih, ail);
+        df_renorm(acc.re.x, acc.re.y);
+        df_renorm(acc.im.x, acc.im.y);
       }
     }
-    re += (double)arh + (double)arl;
-    im += (double)aih + (double)ail;
+    df_renorm(acc.re.x, acc.re.y);
+    df_renorm(acc.im.x, acc.im.y);
   }
 }
 
-// Far terms of coarse cell cc at its node j, one warp: far[cc kCellPC + j].
+// Far terms of coarse cell cc at its node j, one block of kFarThreads:
+// far[cc kCellPC + j].  `red`: one double2 per warp.
+constexpr int kFarThreads = 128;
 template <int FORM>
 __device__ __forceinline__ void cell_far_node(const CellGeom& g, const void* table, const CellTables& T, int cc, int j,
-                                              double2* far) {
-  const int lane = threadIdx.x & 31;
+                                              double2* far, double2* red) {
+  const int tid = threadIdx.x;
   const double C = kCellK * g.c, Xc = (double)(g.k0 + cc * kCellK) * g.w + C;
-  const double x = fma(C, T.coarse_t[j], Xc);
+  const CellX<FORM> x = cell_x<FORM>(g, fma(C, T.coarse_t[j], Xc));
   int lo, hi;
   cell_near(g, cc, lo, hi);
-  double re = 0.0, im = 0.0;
-  // the two far runs as one sequence, so that the lanes share them evenly
+  CellAcc<FORM> acc;
+  // the two far runs as one sequence, so that the threads share them evenly
   const int nfar = lo + g.nterms - hi, skip = hi - lo;
-  const int cut = lo > lane ? (lo - lane + 31) / 32 * 32 + lane : lane;  // first of this lane's indices >= lo
-  cell_terms<FORM>(g, table, x, lane, lo, 32, re, im);
-  cell_terms<FORM>(g, table, x, cut + skip, nfar + skip, 32, re, im);
+  const int cut = lo > tid ? (lo - tid + kFarThreads - 1) / kFarThreads * kFarThreads + tid : tid;  // first index >= lo
+  cell_terms<FORM>(g, table, x, tid, lo, kFarThreads, acc);
+  cell_terms<FORM>(g, table, x, cut + skip, nfar + skip, kFarThreads, acc);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    re += __shfl_xor_sync(0xffffffffu, re, o);
-    im += __shfl_xor_sync(0xffffffffu, im, o);
+    acc.re = cell_add(acc.re, cell_xor(acc.re, o));
+    acc.im = cell_add(acc.im, cell_xor(acc.im, o));
   }
-  if (lane == 0) far[(size_t)cc * kCellPC + j] = make_double2(re, im);
+  if ((tid & 31) == 0) red[tid >> 5] = make_double2(cell_f64(acc.re), cell_f64(acc.im));
+  __syncthreads();
+  if (tid == 0) {
+    double2 s = red[0];
+#pragma unroll
+    for (int w = 1; w < kFarThreads / 32; ++w) s = make_double2(s.x + red[w].x, s.y + red[w].y);
+    far[(size_t)cc * kCellPC + j] = s;
+  }
 }
 
-// Polynomial of one cell, a block of kCellP x 16 threads: 16 lanes per node
-// share the near terms, then the same 16 lanes form the two matrix products.
+// Polynomial of one cell, a block of LANES kCellP threads: the LANES lanes of a
+// node share its near terms; then one warp, (node, re/im) per thread, adds the
+// far values and forms the two matrix products.  That part is in FP64, so it
+// is kept to one warp's instructions (about 80; at 50 in each of the block's
+// warps it took as long as the terms).  DF: coefficients as double-float pairs
+// (float4), else double2.
 template <int FORM>
+struct CellShared {
+  CellX<FORM> x[kCellP];
+  double near[2 * kCellP], f[2 * kCellP], ch[2 * kCellP];
+};
+template <int FORM, bool DF, int LANES>
 __device__ __forceinline__ void cell_poly(const CellGeom& g, const void* table, const CellTables& T, int cell,
-                                          const double2* far, double2* poly, double2* sh /* 2 kCellP */) {
-  const int lane = threadIdx.x & 15, node = threadIdx.x >> 4;
+                                          const double2* far, void* poly, CellShared<FORM>& sh) {
+  const int tid = threadIdx.x, node = tid / LANES, lane = tid % LANES;
   const int cc = cell / kCellK, in = cell - cc * kCellK;
-  const double x = fma(g.c, T.node_t[node], ((double)(g.k0 + cell) + 0.5) * g.w);
+  if (tid < kCellP)
+    sh.x[tid] = cell_x<FORM>(g, fma(g.c, T.node_t[tid], ((double)(g.k0 + cell) + 0.5) * g.w));
   int lo, hi;
   cell_near(g, cc, lo, hi);
-  double re = 0.0, im = 0.0;
-  cell_terms<FORM>(g, table, x, lo + lane, hi, 16, re, im);
+  __syncthreads();
+  CellAcc<FORM> acc;
+  cell_terms<FORM>(g, table, sh.x[node], lo + lane, hi, LANES, acc);
+  // lanes with bit 2 set keep the imaginary part, the others the real part
+  const int comp = (lane >> 2) & 1;
+  auto mine = comp ? acc.im : acc.re;
+  mine = cell_add(mine, cell_xor(comp ? acc.re : acc.im, 4));
+  mine = cell_add(mine, cell_xor(mine, 1));
+  mine = cell_add(mine, cell_xor(mine, 2));
+#pragma unroll
+  for (int o = 8; o < LANES; o *= 2) mine = cell_add(mine, cell_xor(mine, o));
+  if (lane == 0 || lane == 4) {
+    if constexpr (FORM == 0)
+      sh.near[2 * node + comp] = mine;
+    else
+      reinterpret_cast<float2*>(sh.near)[2 * node + comp] = mine;
+  }
+  __syncthreads();
+  if (tid >= 32) return;
+  const int i = tid >> 1, re_im = tid & 1;
+  double a = 0.0, b = 0.0;
+  if constexpr (FORM == 0)
+    a = sh.near[tid];
+  else
+    a = df_to_double(reinterpret_cast<const float2*>(sh.near)[tid]);
   if (g.two_level) {
-    const double* row = T.spread + (size_t)(in * kCellP + node) * kCellPC;
-    const double2* F = far + (size_t)cc * kCellPC;
+    const double2* row = reinterpret_cast<const double2*>(T.spread + (size_t)(in * kCellP + i) * kCellPC);
+    const double* F = reinterpret_cast<const double*>(far + (size_t)cc * kCellPC) + re_im;
 #pragma unroll
-    for (int j = lane; j < kCellPC; j += 16) {
-      const double2 v = F[j];
-      re = fma(row[j], v.x, re);
-      im = fma(row[j], v.y, im);
+    for (int j = 0; j < kCellPC / 2; ++j) {
+      const double2 m = row[j];
+      a = fma(m.x, F[4 * j], a);
+      b = fma(m.y, F[4 * j + 2], b);
     }
   }
-  auto sum16 = [](double& a, double& b) {
+  sh.f[tid] = a + b;
+  __syncwarp();
+  // Chebyshev coefficient i, then the coefficient of t^i
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) {
-      a += __shfl_xor_sync(0xffffffffu, a, o);
-      b += __shfl_xor_sync(0xffffffffu, b, o);
+  for (int step = 0; step < 2; ++step) {
+    const double2* m = reinterpret_cast<const double2*>((step == 0 ? T.to_cheb : T.to_mono) + i * kCellP);
+    const double* f = (step == 0 ? sh.f : sh.ch) + re_im;
+    a = b = 0.0;
+#pragma unroll
+    for (int j = 0; j < kCellP / 2; ++j) {
+      const double2 mj = m[j];
+      a = fma(mj.x, f[4 * j], a);
+      b = fma(mj.y, f[4 * j + 2], b);
     }
-  };
-  sum16(re, im);
-  if (lane == 0) sh[node] = make_double2(re, im);
-  __syncthreads();
-  {  // Chebyshev coefficient `node`
-    const double m = T.to_cheb[node * kCellP + lane];
-    const double2 v = sh[lane];
-    re = m * v.x;
-    im = m * v.y;
-    sum16(re, im);
-    if (lane == 0) sh[kCellP + node] = make_double2(re, im);
+    a += b;
+    if (step == 0) {
+      sh.ch[tid] = a;
+      __syncwarp();
+    }
   }
-  __syncthreads();
-  {  // coefficient of t^node
-    const double m = T.to_mono[node * kCellP + lane];
-    const double2 v = sh[kCellP + lane];
-    re = m * v.x;
-    im = m * v.y;
-    sum16(re, im);
-    if (lane == 0) poly[(size_t)cell * kCellP + node] = make_double2(re, im);
-  }
+  if (DF)
+    static_cast<float2*>(poly)[(size_t)cell * 2 * kCellP + tid] = df_from_double(a);
+  else
+    static_cast<double*>(poly)[(size_t)cell * 2 * kCellP + tid] = a;
 }
 
-// R+(x) from its cell's polynomial.
-__device__ __forceinline__ double2 cell_eval(const CellGeom& g, const double2* __restrict__ poly, double x) {
-  int k = (int)floor(x * g.inv_w) - g.k0;
-  k = min(max(k, 0), g.ncell - 1);  // x beyond the range by rounding: the edge cell's polynomial
-  const double t = (x - ((double)(g.k0 + k) + 0.5) * g.w) * g.inv_c;
-  const double2* p = poly + (size_t)k * kCellP;
+// omega and 1 / omega (0 and 0 at omega = 0) of orbit o.  On the C grid from
+// omega^2 by the hardware's approximate FP64 reciprocal root and a cubic
+// correction, then one residual step for omega: 17 FP64 instructions where
+// the library root and a division take about 45.
+template <bool CGRID>
+__device__ __forceinline__ double2 orbit_omega(const SymbolParams& sp, const OrbitParams& op, int o) {
+  int a, b;
+  orbit_rep(op, o, a, b);
+  if (CGRID) {
+    const double2 hx = sp.half_x[a], hy = sp.half_y[b];
+    const double ax = hx.y * (2.0 * sp.inv_dx), ay = hy.y * (2.0 * sp.inv_dy);
+    const double fc = sp.f * hx.x * hy.x;
+    const double w2 = fma(sp.g * sp.H, fma(ax, ax, ay * ay), fc * fc);
+    if (w2 > 1e-280 && w2 < 1e280) {
+      double y0;
+      asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(w2));
+      const double e = fma(-w2 * y0, y0, 1.0);
+      const double y = fma(y0 * e, fma(0.375, e, 0.5), y0);
+      const double s = w2 * y;
+      return make_double2(fma(fma(-s, s, w2), 0.5 * y, s), y);
+    }
+  }
+  const double w = symbol_at(sp, a, b).omega;
+  return make_double2(w, w > 0.0 ? 1.0 / w : 0.0);
+}
+
+// The cell of x and the local variable t in [-1, 1] (exact: w is a power of two).
+__device__ __forceinline__ int cell_of(const CellGeom& g, double x, double& t) {
+  const double magic = 6755399441055744.0;  // 1.5 2^52: the sum's low bits are the nearest integer
+  const double v = fma(x, g.inv_w, -0.5);
+  const double r = v + magic;
+  double kf = r - magic;
+  int k = __double2loint(r) - g.k0;
+  if (k < 0 || k >= g.ncell) {  // beyond the range by rounding: the edge cell's polynomial
+    k = k < 0 ? 0 : g.ncell - 1;
+    kf = (double)(g.k0 + k);
+  }
+  t = 2.0 * (v - kf);
+  return k;
+}
+
+// fin[o] of orbit o from its cell's polynomial.
+template <int KIND, bool CGRID>
+__device__ __forceinline__ void cell_orbit(const CellGeom& g, const void* __restrict__ poly, const SymbolParams& sp,
+                                           const OrbitParams& op, double tau, double2 R0, int o, void* fin) {
+  const double2 om = orbit_omega<CGRID>(sp, op, o);
+  double t;
+  const int k = cell_of(g, tau * om.x, t);
+  if (KIND == kOrbitDf) {
+    // Horner's rule: the upper half of the coefficients (at most 10.36^-8 =
+    // 7e-9 of the result) in FP32, the lower half in double-float
+    const float4* p = static_cast<const float4*>(poly) + (size_t)k * kCellP;
+    const float2 td = df_from_double(t);
+    float hr = p[kCellP - 1].x, hi = p[kCellP - 1].z;
+#pragma unroll
+    for (int i = kCellP - 2; i >= kCellP / 2; --i) {
+      const float4 v = p[i];
+      hr = fmaf(hr, td.x, v.x);
+      hi = fmaf(hi, td.x, v.z);
+    }
+    float2 ar = make_float2(hr, 0.f), ai = make_float2(hi, 0.f);
+#pragma unroll
+    for (int i = kCellP / 2 - 1; i >= 0; --i) {
+      const float4 v = p[i];
+      const float2 pr = f_mul(ar.x, ar.y, td.x, td.y), pi = f_mul(ai.x, ai.y, td.x, td.y);
+      ar = f_add(v.x, v.y, pr.x, pr.y);
+      ai = f_add(v.z, v.w, pi.x, pi.y);
+    }
+    const float2 iw = df_from_double(om.y);
+    const float2 d = f_subf(df_from_double(R0.x), ar);
+    OrbitScalarsDF out;
+    out.s1 = f_mulf(ai, iw);
+    out.s2 = f_mulf(f_mulf(d, iw), iw);
+    static_cast<OrbitScalarsDF*>(fin)[o] = out;
+    return;
+  }
+  const double2* p = static_cast<const double2*>(poly) + (size_t)k * kCellP;
   double2 a = p[kCellP - 1];
 #pragma unroll
   for (int i = kCellP - 2; i >= 0; --i) {
@@ -165,7 +311,16 @@ __device__ __forceinline__ double2 cell_eval(const CellGeom& g, const double2* _
     a.x = fma(a.x, t, v.x);
     a.y = fma(a.y, t, v.y);
   }
-  return a;
+  if (KIND == kOrbitRaw) {
+    static_cast<double2*>(fin)[o] = a;
+    return;
+  }
+  OrbitScalars out;
+  out.s1 = a.y * om.y;
+  out.s2re = (R0.x - a.x) * om.y * om.y;
+  out.s2im = R0.y * om.y * om.y;
+  out.pad = 0.0;
+  static_cast<OrbitScalars*>(fin)[o] = out;
 }
 
 }  // namespace rexi
