@@ -250,27 +250,31 @@ rexi_status rexi_plan_set_krylov(rexi_plan_t plan, double rtol, int32_t max_iter
  * REXI_KRYLOV_CG (default): one pole-pair CG solve per REXII term, terms
  *   batched (pair operator (alpha_{-n} - dt A)(alpha_n + dt A), Section 3's
  *   reduced sum); computes in the plan's form.
- * REXI_KRYLOV_SHARED: one Lanczos basis of K = -i dt A (self-adjoint in the
- *   energy inner product) shared by every single-shift pole z_j of the step:
- *   (dt A - z_j)^{-1} f = -i (K + i z_j)^{-1} f, and the Krylov space of a
- *   shifted system does not depend on the shift.  Every pole's residual is a
- *   multiple of the next Lanczos vector, so the error of the whole step is
- *   ||f|| b_k phi(K) v_k for a rational function phi known from the Lanczos
+ * REXI_KRYLOV_SHARED: one basis of the Krylov space of K = -i dt A
+ *   (self-adjoint in the energy inner product) shared by every single-shift
+ *   pole z_j of the step: (dt A - z_j)^{-1} f = -i (K + i z_j)^{-1} f, and the
+ *   Krylov space of a shifted system does not depend on the shift.  rtol and
+ *   max_iters are those of rexi_plan_set_krylov: a bound on the error of the
+ *   whole step relative to ||f|| in the energy norm, and a cap on the steps.
+ *   All terms together: Chebyshev polynomials of K on [-dt rho, dt rho], the
+ *   coefficients those of the pole sum, their tail (1e-14) the error bound;
+ *   workspace beyond rexi_workspace_size is not used.  Otherwise (a range of
+ *   terms, rtol below 1e-13, a degree above max_iters, h above about 1, a rho
+ *   set below the plan's own, values near the limits of the arithmetic) Lanczos
+ *   vectors: every pole's residual is a multiple of the next one, so the error
+ *   is ||f|| b_k phi(K) v_k for a rational function phi known from the Lanczos
  *   scalars; the solver stops when b_k max |phi| over [-dt rho, dt rho]
- *   (sampled, rho the plan's spectral radius) is <= rtol (from
- *   rexi_plan_set_krylov, relative to ||f|| in the energy norm; max_iters
- *   caps the Lanczos steps), then forms sum_j beta_j x_j = V_k c.  Lanczos
- *   vectors that fit in workspace bytes beyond rexi_workspace_size (3 nx ny
- *   complex values, or 3 nx ny real values for real input, rounded up to 256
- *   bytes, each) are kept from the first pass; the rest are regenerated from
- *   the stored scalars.  Real input runs the real form of the recurrence
- *   (the vectors alternate between real and imaginary, a_j = 0); in the
- *   mixed form its vectors and stencil arithmetic are double-float (pairs of
- *   FP32 values, about 48 significant bits) with FP64 scalars and inner
- *   products.  FP64 otherwise.  Applies to rexi_step and rexi_step_adjoint,
- *   and, for real input, to rexi_step_grad_depth: two Lanczos runs (on the
- *   input and on W^{-1} grad_out), every vector kept, and the gradient as a
- *   two-sided Galerkin form over the two bases (FP64; workspace from
+ *   (sampled, rho the plan's spectral radius) is <= rtol, then forms
+ *   sum_j beta_j x_j = V_k c.  Lanczos vectors that fit in workspace bytes
+ *   beyond rexi_workspace_size (3 nx ny complex values, or 3 nx ny real values
+ *   for real input, rounded up to 256 bytes, each) are kept from the first
+ *   pass; the rest are regenerated from the stored scalars.
+ *   Real input runs real vectors, in the mixed form double-float ones (pairs
+ *   of FP32 values, about 48 significant bits); FP64 otherwise.  Applies to
+ *   rexi_step and rexi_step_adjoint, and, for real input, to
+ *   rexi_step_grad_depth (same choice of basis: a forward Chebyshev pass that
+ *   keeps one scalar field per step and an adjoint one that consumes them, or
+ *   a two-sided Galerkin form over two kept Lanczos bases; workspace from
  *   rexi_workspace_size_grad_depth, about 2 (3 tau rho + 100) state-sized
  *   real vectors).  Complex input keeps per-term CG for the gradient. */
 enum { REXI_KRYLOV_CG = 0, REXI_KRYLOV_SHARED = 1 };

@@ -380,7 +380,7 @@ rexi_status rexi_plan_create(rexi_plan_t* out, int32_t nx, int32_t ny, double Lx
     p->rho_natural = p->rho;
     st = krylov_init(&p->kry, nx, ny, Lx, Ly, g, f, depth, p->Hmean);
     if (st != REXI_OK) { rexi_plan_destroy(p); return st; }
-    p->kry.rho_bound = p->rho_natural;
+    p->kry.rho_bound = p->kry.rho_op = p->rho_natural;
   }
   if (cudaEventCreateWithFlags(&p->staging_done, cudaEventDisableTiming) != cudaSuccess) {
     rexi_plan_destroy(p);

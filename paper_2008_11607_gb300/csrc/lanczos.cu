@@ -1,5 +1,7 @@
 // Variable-depth path, shared-Krylov method: every single-shift pole of the
-// rational approximation uses one Lanczos basis.
+// rational approximation uses one Krylov basis.  Steps over all terms take
+// Chebyshev polynomials as that basis (cheb.cu); ranges of terms and the other
+// calls that cheb_plan declines take the Lanczos vectors below.
 //
 // With K = -i tau A, which is self-adjoint in the energy inner product
 // <a, b>_W = sum (g/H, 1, 1) conj(a) b (A is skew there), each pole term is
@@ -41,6 +43,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "cheb.h"
 #include "dfloat.cuh"
 #include "internal.h"
 #include "krylov.h"
@@ -53,6 +56,10 @@ constexpr int TX = 32, TY = 16, THREADS = 256, HX = TX + 2, HY = TY + 2;
 constexpr int kChunk = 16;         // Lanczos steps between convergence checks
 constexpr int kCoarse = 8;         // coarse check: every 8th sample of the fine grid
 constexpr int kMinScratchPoles = 32;
+// Tails of the Chebyshev form (cheb.cu): each factor of 10 costs three to five
+// steps, so the sums run to rounding instead of to rtol.  The depth gradient
+// weighs coefficient k by up to k.
+constexpr double kChebTarget = 1e-14, kChebGradTarget = 1e-16;
 // Threads per block of the per-pole recurrences (one thread per pole, a
 // chain of dependent FP64 operations each): one warp per block spreads the
 // poles over as many SMs, and so FP64 pipes, as there are warps.
@@ -1043,6 +1050,27 @@ rexi_status lanczos_impl(KrylovSettings* k, double h, int M, const void* in, voi
     return REXI_ENOMEM;
   }
 
+  // every term: the Chebyshev basis (cheb.cu), unless it declines
+  ChebPlan cp;
+  if (term_begin == 0 && term_end == N + 1 && cheb_plan(k, h, M, dt, kChebTarget, &cp) &&
+      cheb_scratch_bytes(cp, N) <= L.min_total - L.part) {
+    char* b = static_cast<char*>(ws);
+    const ChebBuffers cb = {b, b + L.vb, b + 2 * L.vb, b + L.part};
+    double tail = 0.0;
+    const rexi_status st = cheb_step(k, cp, std::is_same<T, float2>::value ? 1 : 0, h, M, in, out, dt, real_input,
+                                     adjoint, cb, s, hooks, &tail);
+    if (st == REXI_OK && info) {
+      memset(info, 0, sizeof(*info));
+      info->N = N;
+      info->n_terms = real_input ? N + 1 : 2 * N + 1;
+      info->n_poles = npc_max;
+      info->krylov_iters = cp.K;
+      info->krylov_max_rel_res = tail;
+      info->krylov_term_iters = cp.K;
+    }
+    if (st != REXI_EUNSUPPORTED) return st;
+  }
+
   // poles z_j and weights beta_j of the selected REXII terms (partial fractions
   // of each term: z = alpha_{-n} with -Gamma P_n, z = -alpha_n with Gamma Q_n)
   TermSet ts;
@@ -1609,6 +1637,25 @@ rexi_status krylov_grad_depth_lanczos(KrylovSettings* k, int form, double h, int
   }
   const int N = M + kL;
   const size_t nk = (size_t)k->nx * k->ny;
+  ChebPlan cp;
+  if (cheb_plan(k, h, M, dt, kChebGradTarget, &cp) && cheb_scratch_bytes(cp, N) <= L.maxslots - L.part &&
+      cp.K <= 3 * L.cap && L.cap >= 2) {
+    char* b = static_cast<char*>(ws);
+    const ChebGradBuffers cb = {b + L.f0, b + L.g0, b + L.basA, b + L.basA + L.vb, b + L.basB, b + L.part};
+    double tail = 0.0;
+    const rexi_status st =
+        cheb_grad(k, cp, form == REXI_FORM_MIXED ? 1 : 0, h, M, f_in, g_out, grad_depth, dt, cb, s, hooks, &tail);
+    if (st == REXI_OK && info) {
+      memset(info, 0, sizeof(*info));
+      info->N = N;
+      info->n_terms = N + 1;
+      info->n_poles = poles_c(M, 1);
+      info->krylov_iters = cp.K;
+      info->krylov_max_rel_res = tail;
+      info->krylov_term_iters = 2 * (int64_t)cp.K;
+    }
+    if (st != REXI_EUNSUPPORTED) return st;
+  }
   // reduced (real-input) pole set: run on f uses shifts i z_j with beta_j, the run
   // on W^{-1} G uses shifts i conj(z_j) with conj(beta_j)
   TermSet ts;
