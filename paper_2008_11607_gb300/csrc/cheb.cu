@@ -19,7 +19,7 @@
 //   b_k = d_k f + 2 B b_{k+1} + b_{k+2},  r(dt A) f = d_0 f + B b_1 + b_2,
 // which keeps two vectors (b_k overwrites b_{k+2}), stores no basis and needs
 // no second pass.  Against the Lanczos form: 13.9 -> 6.7 ms at 1024^2, tau rho =
-// 400 (double-float), 4.35 -> 1.08 ms at 380 x 310, tau rho = 100 (FP64).
+// 400 (double-float), 4.35 -> 0.77 ms at 380 x 310, tau rho = 100 (FP64).
 //
 // Depth gradient: with mu_k the Clenshaw vectors of W^{-1} G for -dt (B^T = -W
 // B W^{-1}), dL = sum_k c'_k <W mu_{k+1}, dB P_k> (c'_0 = 1, else 2), and H
@@ -28,7 +28,7 @@
 // one pass forward that stores the scalar field s_k per step and one Clenshaw
 // pass that consumes them, O(K nk) work where the two-sided Lanczos form
 // contracts K x K pairs of basis vectors (8 steps with gradients at 512^2, tau
-// rho = 200: 269 -> 47 ms).
+// rho = 200: 269 -> 27 ms).
 //
 // Unknowns are scaled, U = (2 dt / (Lh dx)) u, V = (2 dt / (Lh dy)) v, so that
 // the divergence needs no products and each momentum row two.
@@ -235,6 +235,7 @@ struct StepArgs {
   double* grad;      // last: the depth gradient
   const double* w;
   int adjoint, real_out;
+  const unsigned* bad;  // last: nonzero where an earlier launch gave up (the result is then NaN)
 };
 
 // One step of the recurrence on a tile of TX x TY points, two rows per thread.
@@ -279,6 +280,7 @@ __global__ void __launch_bounds__(THREADS, 4) cheb_step_kernel(Geom<T> G, StepAr
   }
   T dk = T{};
   if (!FWD) dk = *A.d;
+  if (LAST && A.bad && *A.bad) dk = u_from<T>(nan(""));
   cp_async_wait_all();
   __syncthreads();
   const T cu = HALF ? u_half(G.cu) : G.cu, gu = HALF ? u_half(G.gu) : G.gu;
@@ -315,7 +317,8 @@ __global__ void __launch_bounds__(THREADS, 4) cheb_step_kernel(Geom<T> G, StepAr
       }
       if (FWD) A.s[id] = u_norm(s);
       if (GRAD) {
-        const T es = LAST ? u_half(e) : e;
+        T es = LAST ? u_half(e) : e;
+        if (LAST && A.bad && *A.bad) es = dk;
         const T t = u_norm(u_madd(A.first ? T{} : A.acc[id], es, ps[r]));
         if (MODE == kGrad)
           A.acc[id] = t;
@@ -345,10 +348,10 @@ __global__ void __launch_bounds__(THREADS, 4) cheb_step_kernel(Geom<T> G, StepAr
   }
 }
 
-// Launch that may overlap the previous step's tail (see pdl_wait); an error is
-// left for the caller's cudaGetLastError.
+// Launch that may overlap the previous step's tail (see pdl_wait; not behind a
+// launch of many steps, which wrote what this one loads early); an error is left for the caller's cudaGetLastError.
 template <typename T, int MODE>
-void launch_step(const Geom<T>& G, const StepArgs<T>& A, int nset, cudaStream_t s) {
+void launch_step(const Geom<T>& G, const StepArgs<T>& A, int nset, cudaStream_t s, bool overlap = true) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((G.nx + TX - 1) / TX, (G.ny + TY - 1) / TY, nset);
   cfg.blockDim = dim3(THREADS);
@@ -357,8 +360,409 @@ void launch_step(const Geom<T>& G, const StepArgs<T>& A, int nset, cudaStream_t 
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = overlap ? 1 : 0;
   cudaLaunchKernelEx(&cfg, cheb_step_kernel<T, MODE>, G, A);
+}
+
+// ---- many steps in one launch ------------------------------------------------
+//
+// Steps on grids whose vectors fit the multiprocessors' shared memory: every
+// block keeps a tile (b_{k+1}, b_{k+2}, F, H with a halo) there for all steps and
+// passes only its edge values to its neighbours.  An edge value travels through
+// L2 as two 64-bit words, each 32 bits of it and the step's number, so that the
+// reader polls the value itself: no flag and no fence on the way.  The tile's
+// edge is computed first; while the compute warps work on the interior, the
+// last kCommWarps warps publish the edge, poll the neighbours' and fill the next
+// step's halo, so a step costs the longer of the two.  Two slots per edge
+// value, by the parity of the step: a block overwrites a slot only after it has
+// the next step's edges of every reader (west / east, south / north and the two
+// corners that the Coriolis averages touch are neighbours in both directions).
+// A launch per step costs 2.2 us however small the grid, and moves 13 values per
+// point through L2.  Per step, one launch each -> tiles: 512^2 double-float 4.93
+// -> 2.54 us, 256^2 2.47 -> 1.73, 96 x 80 2.56 -> 1.7; 380 x 310 FP64 7.36 -> 5.2
+// (FP64 pipe: 3.8 us at its peak rate), 100 x 90 4.49 -> 2.4.  What is left at
+// 512^2 is issue (3.15 of 4 instructions per cycle, 224 of 332 per point on the
+// FMA pipe before a task took two rows); below 256^2 it is the way of an edge
+// value through L2, 1.2 us.
+struct Exchange {
+  ulonglong2 *col, *row;  // [parity][set][3][strip][ny], [parity][set][3][group][nx]
+  unsigned* bad;          // a wait ran out
+};
+enum { kColE = 0, kColV = 1, kColU = 2, kRowE = 0, kRowU = 1, kRowV = 2 };
+
+__device__ __forceinline__ ulonglong2 pack(float2 v, unsigned flag) {
+  const unsigned long long f = (unsigned long long)flag << 32;
+  return make_ulonglong2(f | __float_as_uint(v.x), f | __float_as_uint(v.y));
+}
+__device__ __forceinline__ ulonglong2 pack(double v, unsigned flag) {
+  const unsigned long long f = (unsigned long long)flag << 32;
+  return make_ulonglong2(f | (unsigned)__double2loint(v), f | (unsigned)__double2hiint(v));
+}
+template <typename T>
+__device__ __forceinline__ T unpack(ulonglong2 w);
+template <>
+__device__ __forceinline__ float2 unpack<float2>(ulonglong2 w) {
+  return make_float2(__uint_as_float((unsigned)w.x), __uint_as_float((unsigned)w.y));
+}
+template <>
+__device__ __forceinline__ double unpack<double>(ulonglong2 w) {
+  return __hiloint2double((int)(unsigned)w.y, (int)(unsigned)w.x);
+}
+__device__ __forceinline__ void st_edge(ulonglong2* p, ulonglong2 w) {
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(w.x), "l"(w.y) : "memory");
+}
+__device__ __forceinline__ ulonglong2 ld_edge(const ulonglong2* p) {
+  ulonglong2 w;
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w.x), "=l"(w.y) : "l"(p) : "memory");
+  return w;
+}
+__device__ __forceinline__ bool arrived(ulonglong2 w, unsigned flag) {
+  return (unsigned)(w.x >> 32) == flag && (unsigned)(w.y >> 32) == flag;
+}
+// Polls of one wait before a warp gives up (about a second; a warp's neighbours are
+// resident with it, so a wait lasts microseconds).
+constexpr int kPollLimit = 1 << 20;
+
+template <typename T>
+struct ManyArgs {
+  const T *b1, *b2;  // newest vectors (b2 null: zero)
+  T *o1, *o2;        // where the newest two go at the end (null: nowhere)
+  const T *F, *H, *d;  // d: coefficient of the first step, descending
+  T* s;              // kForward: s of the first step, ascending; kGrad: of the first step, descending
+  T* acc;            // kGrad: sum of mu_eta s (written)
+  int steps, nset, ns, ng, seg_shift;
+  unsigned flag0;    // flags of earlier launches on this exchange buffer end here
+  Exchange X;
+};
+
+constexpr int kCommWarps = 4, kComm = 32 * kCommWarps, kSlots = 4;  // edge values per communicating thread
+constexpr int kMaxComputeWarps = 16;
+
+// A block's tile: W columns by rows rows; a field is kept with pitch P, E and U
+// with rows 0 .. rows, V with rows -1 .. rows - 1, columns -1 .. W.
+struct Tile {
+  int W, rows, P, fs;
+  __device__ int at(int x, int y) const { return y * P + x + 1; }        // in a field of E or U
+  __device__ int atv(int x, int y) const { return 2 * fs + (y + 1) * P + x + 1; }  // V in a vector
+};
+__host__ __device__ inline int tile_pitch(int W) { return (W + 2) | 1; }
+__host__ __device__ inline size_t tile_values(int W, int rows, bool grad) {
+  return (size_t)tile_pitch(W) * (6 * (rows + 1) + (grad ? 5 : 4) * rows);
+}
+
+template <typename T, int MODE>
+__global__ void __launch_bounds__(32 * (kMaxComputeWarps + kCommWarps), 1) cheb_many_kernel(Geom<T> G, ManyArgs<T> A) {
+  constexpr bool FWD = MODE == kForward, GRAD = MODE == kGrad;
+  extern __shared__ double smem_raw[];
+  __shared__ unsigned dead;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nc = (blockDim.x >> 5) - kCommWarps;  // compute warps
+  const int per_set = A.ns * A.ng;
+  const int set = blockIdx.x / per_set, strip = blockIdx.x % per_set / A.ng, grp = blockIdx.x % A.ng;
+  const int nx = G.nx, ny = G.ny;
+  // columns [i0, i0 + W), rows [j0, j0 + rows)
+  const int wq = nx / A.ns, wr = nx % A.ns, hq = ny / A.ng, hr = ny % A.ng;
+  const int i0 = strip * wq + min(strip, wr), j0 = grp * hq + min(grp, hr);
+  Tile t;
+  t.W = wq + (strip < wr);
+  t.rows = hq + (grp < hr);
+  t.P = tile_pitch(t.W);
+  t.fs = (t.rows + 1) * t.P;
+  const int W = t.W, rows = t.rows, fs = t.fs;
+  T* cur = reinterpret_cast<T*>(smem_raw);
+  T* old = cur + 3 * fs;
+  T* sF = old + 3 * fs;            // 3 fields of rows x P
+  T* sH = sF + 3 * rows * t.P;
+  T* sA = sH + rows * t.P;         // the gradient's sum
+  const size_t nk = G.nk, so = (size_t)set * 3 * nk;
+  const size_t id0 = (size_t)j0 * nx + i0;
+  for (int q = threadIdx.x; q < W * rows; q += blockDim.x) {
+    const int x = q % W, y = q / W, a = t.at(x, y), av = t.atv(x, y), f = y * t.P + x;
+    const size_t o = so + id0 + (size_t)y * nx + x;
+    cur[a] = A.b1[o];
+    cur[fs + a] = A.b1[o + nk];
+    cur[av] = A.b1[o + 2 * nk];
+    old[a] = A.b2 ? A.b2[o] : T{};
+    old[fs + a] = A.b2 ? A.b2[o + nk] : T{};
+    old[av] = A.b2 ? A.b2[o + 2 * nk] : T{};
+    if (!FWD) {
+      sF[f] = A.F[o];
+      sF[rows * t.P + f] = A.F[o + nk];
+      sF[2 * rows * t.P + f] = A.F[o + 2 * nk];
+    }
+    sH[f] = u_neg(A.H[o - so]);
+    if (GRAD) sA[f] = T{};
+  }
+  if (threadIdx.x == 0) dead = 0u;
+  __syncthreads();
+
+  if (warp >= nc) {
+    // ---- edges
+    const size_t ncol = (size_t)3 * A.ns * ny, nrow = (size_t)3 * A.ng * nx;
+    const size_t pcol = A.nset * ncol, prow = A.nset * nrow;
+    const int strip_w = strip ? strip - 1 : A.ns - 1, strip_e = strip + 1 < A.ns ? strip + 1 : 0;
+    const int grp_s = grp ? grp - 1 : A.ng - 1, grp_n = grp + 1 < A.ng ? grp + 1 : 0;
+    const int jn = j0 + rows < ny ? j0 + rows : 0, js = j0 ? j0 - 1 : ny - 1;
+    // slot of a column (row) edge value at an even step; an odd step's is a parity
+    // stride further on (odd: the stride, in units of a slot)
+    auto col_slot = [&](int kind, int st, int j) { return (unsigned)(set * ncol + ((size_t)kind * A.ns + st) * ny + j); };
+    auto row_slot = [&](int kind, int g, int i) {
+      return (unsigned)(2 * pcol + set * nrow + ((size_t)kind * A.ng + g) * nx + i);
+    };
+    int src[kSlots], dst[kSlots];            // tile offsets, -1: none
+    unsigned put[kSlots], get[kSlots], podd[kSlots], godd[kSlots];
+#pragma unroll
+    for (int m = 0; m < kSlots; ++m) {
+      const int c = threadIdx.x - 32 * nc;
+      int q = c + kComm * m;
+      src[m] = dst[m] = -1;
+      put[m] = get[m] = 0u;
+      podd[m] = godd[m] = (unsigned)(q < 3 * W ? prow : pcol);
+      if (q < 3 * W) {
+        const int k = q / W, x = q % W;
+        src[m] = k == kRowE ? t.at(x, 0) : (k == kRowU ? fs + t.at(x, 0) : t.atv(x, rows - 1));
+        put[m] = row_slot(k, grp, i0 + x);
+        dst[m] = k == kRowE ? t.at(x, rows) : (k == kRowU ? fs + t.at(x, rows) : t.atv(x, -1));
+        get[m] = row_slot(k, k == kRowV ? grp_s : grp_n, i0 + x);
+        continue;
+      }
+      q -= 3 * W;
+      const int qp = q;
+      if (qp < 3 * rows) {
+        const int k = qp / rows, y = qp % rows;
+        src[m] = k == kColE ? t.at(0, y) : (k == kColV ? t.atv(0, y) : fs + t.at(W - 1, y));
+        put[m] = col_slot(k, strip, j0 + y);
+      }
+      // E rows 0 .., V rows -1 .. of the east strip, U rows 0 .. rows of the west strip
+      if (q < rows) {
+        dst[m] = t.at(W, q);
+        get[m] = col_slot(kColE, strip_e, j0 + q);
+      } else if ((q -= rows) <= rows) {
+        dst[m] = t.atv(W, q - 1);
+        get[m] = col_slot(kColV, strip_e, q ? j0 + q - 1 : js);
+      } else if ((q -= rows + 1) <= rows) {
+        dst[m] = fs + t.at(-1, q);
+        get[m] = col_slot(kColU, strip_w, q < rows ? j0 + q : jn);
+      }
+    }
+    ulonglong2* X = A.X.col;
+    // sends the edge of b under `flag` and fills b's halo with the neighbours'
+    auto exchange = [&](T* b, unsigned flag) {
+#pragma unroll
+      for (int m = 0; m < kSlots; ++m)
+        if (src[m] >= 0) st_edge(X + put[m] + ((flag & 1) ? podd[m] : 0u), pack(b[src[m]], flag));
+      unsigned left = 0;
+#pragma unroll
+      for (int m = 0; m < kSlots; ++m)
+        if (dst[m] >= 0) left |= 1u << m;
+      for (int n = 0; left; ++n) {
+        ulonglong2 w[kSlots];
+#pragma unroll
+        for (int m = 0; m < kSlots; ++m)
+          if (left >> m & 1) w[m] = ld_edge(X + get[m] + ((flag & 1) ? godd[m] : 0u));
+#pragma unroll
+        for (int m = 0; m < kSlots; ++m)
+          if ((left >> m & 1) && arrived(w[m], flag)) {
+            b[dst[m]] = unpack<T>(w[m]);
+            left &= ~(1u << m);
+          }
+        if (n >= kPollLimit || ((n & 1023) == 1023 && *(volatile unsigned*)A.X.bad)) {
+          *(volatile unsigned*)A.X.bad = 1u;
+          *(volatile unsigned*)&dead = 1u;
+          return;
+        }
+      }
+    };
+    exchange(cur, A.flag0 + 1);
+    __syncthreads();
+    for (int step = 0; step < A.steps; ++step) {
+      if (*(volatile unsigned*)&dead) return;
+      asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");  // the edge is computed
+      if (step + 1 < A.steps) exchange(old, A.flag0 + 2 + step);
+      T* x = cur;
+      cur = old;
+      old = x;
+      __syncthreads();
+    }
+    return;
+  }
+
+  // ---- points: the first and last row, then the outer columns, then the rest
+  const int sh = A.seg_shift, seg = 1 << sh, inner = max(rows - 2, 0);  // seg: warps to a row of the widest tile
+  const int t_row = (rows > 1 ? 2 : 1) * seg, t_col = (2 * inner + 31) / 32, t_all = t_row + t_col + (inner + 1) / 2 * seg;
+  __syncthreads();
+  for (int step = 0; step < A.steps; ++step) {
+    if (*(volatile unsigned*)&dead) return;
+    T dk = T{};
+    if (!FWD) dk = A.d[-step];
+    bool told = false;
+    for (int k = warp; k < t_all; k += nc) {
+      if (!told && k >= t_row + t_col) {
+        told = true;
+        asm volatile("bar.arrive 1, %0;" ::"r"(blockDim.x) : "memory");
+      }
+      int x, y;
+      bool live, two = false;
+      if (k < t_row) {
+        x = (k & (seg - 1)) * 32 + lane;
+        y = k < seg ? 0 : rows - 1;
+        live = x < W;
+      } else if (k < t_row + t_col) {
+        const int q = (k - t_row) * 32 + lane;
+        live = q < 2 * inner;
+        x = q < inner ? 0 : W - 1;
+        y = 1 + (q < inner ? q : q - inner);
+      } else {
+        const int q = k - t_row - t_col;
+        x = (q & (seg - 1)) * 32 + lane;
+        y = 1 + 2 * (q >> sh);
+        two = y + 1 < rows - 1;
+        live = x > 0 && x < W - 1;
+      }
+      if (!live) x = y = 0;
+      const T* c = cur + t.at(x, y);
+      const T* v = cur + t.atv(x, y);
+      T* b = old + t.at(x, y);
+      T* bv = old + t.atv(x, y);
+      int f = y * t.P + x;
+      size_t o = id0 + (size_t)y * nx + x;
+      // carried from row to row: E, U's difference and pair sum, V below and its pair sum
+      T e = c[0], u = c[fs], w = c[fs - 1], vs = v[-t.P];
+      T ps[2] = {};
+      if (GRAD) {
+        const T* sp = A.s - (size_t)step * nk + o;
+        ps[0] = sp[0];
+        if (two) ps[1] = sp[nx];
+      }
+      T du = u_sub(u, w), su = u_add(u, w), sv = u_add(vs, v[1 - t.P]);
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        if (r == 1 && !two) break;
+        const T vo = v[0], svn = u_add(vo, v[1]), en = c[t.P];
+        u = c[fs + t.P];
+        w = c[fs + t.P - 1];
+        T a0 = b[0], a1 = b[fs], a2 = bv[0];
+        if (!FWD) {
+          a0 = u_madd(a0, sF[f], dk);
+          a1 = u_madd(a1, sF[rows * t.P + f], dk);
+          a2 = u_madd(a2, sF[2 * rows * t.P + f], dk);
+        }
+        const T s = u_add(du, u_sub(vo, vs)), sun = u_add(u, w);
+        a0 = u_norm(u_madd(a0, s, sH[f]));
+        a1 = u_madd(a1, u_add(sv, svn), G.cu);
+        a1 = u_norm(u_madd(a1, u_sub(c[1], e), u_neg(G.gu)));
+        a2 = u_madd(a2, u_add(su, sun), u_neg(G.cv));
+        a2 = u_norm(u_madd(a2, u_sub(en, e), u_neg(G.gv)));
+        if (live) {
+          b[0] = a0;
+          b[fs] = a1;
+          bv[0] = a2;
+          if (FWD) A.s[o + (size_t)step * nk] = u_norm(s);
+          if (GRAD) sA[f] = u_norm(u_madd(sA[f], e, ps[r]));
+        }
+        if (r == 0) {
+          e = en;
+          du = u_sub(u, w);
+          su = sun;
+          sv = svn;
+          vs = vo;
+          c += t.P;
+          v += t.P;
+          b += t.P;
+          bv += t.P;
+          f += t.P;
+          o += nx;
+        }
+      }
+    }
+    if (!told) asm volatile("bar.arrive 1, %0;" ::"r"(blockDim.x) : "memory");
+    T* x = cur;
+    cur = old;
+    old = x;
+    __syncthreads();
+  }
+  for (int q = threadIdx.x; q < W * rows; q += 32 * nc) {
+    const int x = q % W, y = q / W, a = t.at(x, y), av = t.atv(x, y);
+    const size_t o = so + id0 + (size_t)y * nx + x;
+    if (A.o1) {
+      A.o1[o] = cur[a];
+      A.o1[o + nk] = cur[fs + a];
+      A.o1[o + 2 * nk] = cur[av];
+      A.o2[o] = old[a];
+      A.o2[o + nk] = old[fs + a];
+      A.o2[o + 2 * nk] = old[av];
+    }
+    if (GRAD) A.acc[o - so] = sA[y * t.P + x];
+  }
+}
+
+size_t exchange_bytes(int ns, int ng, int nx, int ny, int nset) {
+  return 256 + (size_t)2 * nset * 3 * ((size_t)ns * ny + (size_t)ng * nx) * sizeof(ulonglong2);
+}
+// The tiles for a grid, one block per multiprocessor, or blocks == 0 where they do
+// not fit: of the ways to cut the grid into ns strips of ng tiles, the one
+// whose blocks have the fewest warp-rows to compute, then the fewest edge values.
+struct ManyPlan {
+  int ns = 0, ng = 0, blocks = 0, warps = 0, seg_shift = 0;  // warps: compute warps; 2^seg_shift warps to a row
+  size_t smem = 0;
+};
+ManyPlan many_plan(int nx, int ny, int nset, int sms, bool grad, size_t exchange) {
+  ManyPlan p;
+  long long best = 1ll << 62;
+  for (int ns = 1; ns * nset <= sms && 2 * ns <= nx; ++ns) {
+    const int top = std::min(sms / (ns * nset), ny), W = (nx + ns - 1) / ns, H = (ny + top - 1) / top;
+    const int ng = (ny + H - 1) / H;  // no more tiles than rows of height H need
+    int sh = 0;
+    while (32 << sh < W) ++sh;
+    const int seg = 1 << sh, inner = std::max(H - 2, 0);
+    const int edge = (H > 1 ? 2 : 1) * seg + (2 * inner + 31) / 32, tasks = edge + (inner + 1) / 2 * seg;
+    const int work = seg * H + (2 * inner + 31) / 32;
+    const size_t smem = tile_values(W, H, grad) * 8;
+    if (3 * W + 3 * H + 2 > kComm * kSlots || smem > 226 * 1024 || exchange_bytes(ns, ng, nx, ny, nset) > exchange)
+      continue;
+    const long long c = (long long)work * 4096 + W + H;
+    if (c >= best) continue;
+    best = c;
+    p.ns = ns;
+    p.ng = ng;
+    p.blocks = ns * ng * nset;
+    // two turns or more where most of the work is inside, so that the edge is not
+    // computed in step with the rest (256^2: 2.10 -> 1.73 us per step)
+    const int turns = std::max(2 * edge <= tasks ? 2 : 1, (tasks + kMaxComputeWarps - 1) / kMaxComputeWarps);
+    p.warps = (tasks + turns - 1) / turns;
+    p.seg_shift = sh;
+    p.smem = smem;
+  }
+  return p;
+}
+cudaError_t exchange_at(const ManyPlan& p, int nx, int ny, int nset, void* base, Exchange* X, cudaStream_t s) {
+  char* b = static_cast<char*>(base);
+  X->bad = reinterpret_cast<unsigned*>(b);
+  X->col = reinterpret_cast<ulonglong2*>(b + 256);
+  X->row = X->col + (size_t)2 * nset * 3 * p.ns * ny;
+  return cudaMemsetAsync(b, 0, exchange_bytes(p.ns, p.ng, nx, ny, nset), s);
+}
+template <typename T, int MODE>
+cudaError_t launch_many(const Geom<T>& G, ManyArgs<T> A, const ManyPlan& p, int nset, cudaStream_t s, bool* launched) {
+  A.nset = nset;
+  A.ns = p.ns;
+  A.ng = p.ng;
+  A.seg_shift = p.seg_shift;
+  auto kern = cheb_many_kernel<T, MODE>;
+  Geom<T> geom = G;
+  void* args[] = {&geom, &A};
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+  if (e == cudaSuccess)
+    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kern), dim3(p.blocks),
+                                    dim3(32 * (p.warps + kCommWarps)), args, p.smem, s);
+  // a device that cannot hold the grid at once (part of it set aside): one
+  // launch per step
+  *launched = e == cudaSuccess;
+  if (e == cudaErrorCooperativeLaunchTooLarge) {
+    cudaGetLastError();
+    return cudaSuccess;
+  }
+  return e;
 }
 
 // Smallest K with 2 sum_{k > K} |J_k(x)| <= target: Miller's downward
@@ -533,8 +937,30 @@ rexi_status step_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
   A.F = F;
   A.H = depth_table(k, T{});
   const T *b1, *b2;
-  clenshaw<T, kSum>(G, A, p.K, d, bA, bB, nullptr, nset, s, &b1, &b2);
-  launches += p.K - 1;
+  const ManyPlan mp = many_plan(k->nx, k->ny, nset, k->sms, false, b.exchange_bytes);
+  bool many = mp.blocks && p.K > 2;
+  if (many) {
+    ManyArgs<T> Q = {};
+    e = exchange_at(mp, k->nx, k->ny, nset, b.exchange, &Q.X, s);
+    Q.b1 = bA;
+    Q.o1 = bA;
+    Q.o2 = bB;
+    Q.F = F;
+    Q.H = A.H;
+    Q.d = d + p.K - 1;
+    Q.steps = p.K - 1;
+    if (e == cudaSuccess) e = launch_many<T, kSum>(G, Q, mp, nset, s, &many);
+    if (e != cudaSuccess) return failed(e);
+    b1 = bA;
+    b2 = bB;
+    A.bad = Q.X.bad;
+    launches += many;
+  }
+  if (!many) {
+    A.bad = nullptr;
+    clenshaw<T, kSum>(G, A, p.K, d, bA, bB, nullptr, nset, s, &b1, &b2);
+    launches += p.K - 1;
+  }
   mark(2);
   mark(3);
   // the host looks at the tail and the input while the steps run; `out` is
@@ -550,7 +976,7 @@ rexi_status step_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
     A.w = k->w64;
     A.adjoint = adjoint ? 1 : 0;
     A.real_out = real_input;
-    launch_step<T, kSumLast>(G, A, nset, s);
+    launch_step<T, kSumLast>(G, A, nset, s, !many);
     ++launches;
   }
   mark(4);
@@ -577,6 +1003,12 @@ rexi_status grad_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
   mark(0);
   cudaError_t e = coefficients(p, h, M, S, s, &launches);
   mark(1);
+  const ManyPlan mp = many_plan(k->nx, k->ny, 1, k->sms, true, b.exchange_bytes);
+  bool many = mp.blocks && p.K > 2;
+  ManyArgs<T> Q = {};
+  Q.H = depth_table(k, T{});
+  Q.steps = p.K - 1;
+  if (many && e == cudaSuccess) e = exchange_at(mp, k->nx, k->ny, 1, b.exchange, &Q.X, s);
   // forward: P_0 in bA, P_1 in bB, then each P_{k+1} over P_{k-1}; s_k for k < K
   Geom<T> G = make_geom<T>(k, dt, p);
   if (e == cudaSuccess) e = init(G, k, f_in, 0, bA, static_cast<T*>(nullptr), d, S, 1, s, &launches);
@@ -595,10 +1027,19 @@ rexi_status grad_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
         launch_step<T, kForwardFirst>(G, A, 1, s);
       else
         launch_step<T, kForward>(G, A, 1, s);
+      ++launches;
       std::swap(cur, old);
+      if (j == 0 && many) {
+        Q.b1 = cur;
+        Q.b2 = old;
+        Q.s = sf + G.nk;
+        e = launch_many<T, kForward>(G, Q, mp, 1, s, &many);
+        if (e != cudaSuccess) return failed(e);
+        launches += many;
+        if (many) break;
+      }
     }
   }
-  launches += p.K;
   // backward: the Clenshaw vectors of W^{-1} G under -dt, each step taking its s_k
   G = make_geom<T>(k, -dt, p);
   e = init(G, k, g_out, 1, F, bA, d + p.K, S, 1, s, &launches);
@@ -610,8 +1051,28 @@ rexi_status grad_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
   A.acc = static_cast<T*>(b.acc);
   A.first = 1;
   const T *b1, *b2;
-  clenshaw<T, kGrad>(G, A, p.K, d, bA, bB, sf, 1, s, &b1, &b2);
-  launches += p.K - 1;
+  if (many) {
+    Q.b1 = bA;
+    Q.b2 = nullptr;
+    Q.o1 = bA;
+    Q.o2 = bB;
+    Q.F = F;
+    Q.d = d + p.K - 1;
+    Q.s = sf + (size_t)(p.K - 1) * G.nk;
+    Q.acc = A.acc;
+    Q.flag0 = p.K;
+    e = launch_many<T, kGrad>(G, Q, mp, 1, s, &many);
+    if (e != cudaSuccess) return failed(e);
+    b1 = bA;
+    b2 = bB;
+    A.bad = Q.X.bad;
+    launches += many;
+  }
+  if (!many) {
+    A.bad = nullptr;
+    clenshaw<T, kGrad>(G, A, p.K, d, bA, bB, sf, 1, s, &b1, &b2);
+    launches += p.K - 1;
+  }
   mark(2);
   mark(3);
   bool okf = false, okg = false;
@@ -626,7 +1087,7 @@ rexi_status grad_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
     A.s = sf;
     A.grad = grad_depth;
     A.w = k->w64;
-    launch_step<T, kGradLast>(G, A, 1, s);
+    launch_step<T, kGradLast>(G, A, 1, s, !many);
     ++launches;
   }
   mark(4);

@@ -25,6 +25,8 @@ size_t cheb_scratch_bytes(const ChebPlan& p, int N);
 struct ChebBuffers {
   void *f0, *bA, *bB;  // state-sized vectors (nset x 3 nk values of 8 bytes)
   void* scratch;       // cheb_scratch_bytes
+  void* exchange;      // edge values between warps (any size; 256-byte aligned)
+  size_t exchange_bytes;
 };
 // out = r(dt A) in (adjoint: r(dt A)^H), as krylov_step.  REXI_EUNSUPPORTED,
 // with `out` untouched, where the input or the coefficients call for the
@@ -38,6 +40,8 @@ struct ChebGradBuffers {
   void* acc;           // nk values of 8 bytes
   void* div;           // K nk values of 8 bytes
   void* scratch;       // cheb_scratch_bytes
+  void* exchange;      // edge values between warps (any size; 256-byte aligned)
+  size_t exchange_bytes;
 };
 // grad_depth += dL/dH for out = r(dt A(H)) f_in, G = dL/d out (real input);
 // same refusals, with grad_depth untouched.

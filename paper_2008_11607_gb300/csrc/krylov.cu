@@ -660,6 +660,12 @@ rexi_status krylov_init(KrylovSettings* k, int nx, int ny, double Lx, double Ly,
   k->f = f;
   k->depth = depth;
   k->Hmean = Hmean;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&k->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    set_last_error("device query failed");
+    return REXI_ECUDA;
+  }
   const size_t nk = (size_t)nx * ny;
   char* mem = nullptr;
   const size_t bytes = al256(nk * sizeof(double)) + 2 * al256(nk * sizeof(float)) + 2 * al256(nk * sizeof(float2));

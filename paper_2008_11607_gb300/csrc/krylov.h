@@ -19,6 +19,7 @@ struct KrylovSettings {
   int method = 0;             // 0: CG per REXII term; 1: one Lanczos basis shared by all poles
   double rho_bound = 0;       // upper bound of ||A||_W (the plan's own rho)
   double rho_op = 0;          // the operator's own bound, whatever rho the plan was given
+  int sms = 0;                // multiprocessors of the device
   double* pinned = nullptr;   // small pinned host buffer (convergence checks)
   cudaEvent_t ev[2] = {nullptr, nullptr};
   void* dev_state = nullptr;  // plan-owned device tables below

@@ -1055,7 +1055,7 @@ rexi_status lanczos_impl(KrylovSettings* k, double h, int M, const void* in, voi
   if (term_begin == 0 && term_end == N + 1 && cheb_plan(k, h, M, dt, kChebTarget, &cp) &&
       cheb_scratch_bytes(cp, N) <= L.min_total - L.part) {
     char* b = static_cast<char*>(ws);
-    const ChebBuffers cb = {b, b + L.vb, b + 2 * L.vb, b + L.part};
+    const ChebBuffers cb = {b, b + L.vb, b + 2 * L.vb, b + L.part, b + 3 * L.vb, L.alpha - 3 * L.vb};
     double tail = 0.0;
     const rexi_status st = cheb_step(k, cp, std::is_same<T, float2>::value ? 1 : 0, h, M, in, out, dt, real_input,
                                      adjoint, cb, s, hooks, &tail);
@@ -1639,9 +1639,10 @@ rexi_status krylov_grad_depth_lanczos(KrylovSettings* k, int form, double h, int
   const size_t nk = (size_t)k->nx * k->ny;
   ChebPlan cp;
   if (cheb_plan(k, h, M, dt, kChebGradTarget, &cp) && cheb_scratch_bytes(cp, N) <= L.maxslots - L.part &&
-      cp.K <= 3 * L.cap && L.cap >= 2) {
+      cp.K <= 3 * L.cap && L.cap >= 3) {
     char* b = static_cast<char*>(ws);
-    const ChebGradBuffers cb = {b + L.f0, b + L.g0, b + L.basA, b + L.basA + L.vb, b + L.basB, b + L.part};
+    const ChebGradBuffers cb = {b + L.f0, b + L.g0, b + L.basA, b + L.basA + L.vb,
+                                b + L.basB, b + L.part, b + L.basA + 2 * L.vb, (size_t)(L.cap - 2) * L.vb};
     double tail = 0.0;
     const rexi_status st =
         cheb_grad(k, cp, form == REXI_FORM_MIXED ? 1 : 0, h, M, f_in, g_out, grad_depth, dt, cb, s, hooks, &tail);

@@ -69,6 +69,42 @@ def test_step_adjoint_gradient_at_tile_edges(nx, ny, taurho):
 
 
 @pytest.mark.parametrize("form", ["fp64", "mixed"])
+@pytest.mark.parametrize("nx,ny,real", [(1001, 650, True), (507, 495, False), (640, 343, True)])
+def test_grids_beyond_shared_memory_match_fourier(nx, ny, real, form):
+    """Ragged grids that take one launch per step (the last: the largest that the
+    tiles hold, nearly), with H = 1 against the Fourier path."""
+    torch = torch_cuda()
+    from paper_2008_11607_gb300 import rexi
+
+    st = inputs.complex_random_state(nx, ny, seed=3)
+    if real:
+        st = st.real.astype(np.complex128)
+    plan = _plan(torch, nx, ny, np.ones((ny, nx)), form)
+    dt = 20.0 / plan.rho
+    x = to_dev(torch, st)
+    got = plan.step(x, dt, real_input=real)
+    ref = rexi.Plan(nx, ny).step(x, dt, real_input=real)
+    assert rel_l2(got.cpu().numpy(), ref.cpu().numpy()) < _tol(form, np.ones(1))
+
+
+@pytest.mark.parametrize("form", ["fp64", "mixed"])
+def test_gradient_beyond_shared_memory_matches_lanczos(form):
+    """The depth gradient at 701 x 650 (one launch per step) against the two-sided
+    Lanczos form, which a bound below 1e-13 selects; the tolerance of the
+    gradient's oracle tests."""
+    torch = torch_cuda()
+    nx, ny = 701, 650
+    H = inputs.variable_depth(nx, ny, seed=5)
+    x = to_dev(torch, inputs.kminus3_field(nx, ny, seed=6))
+    G = to_dev(torch, inputs.kminus3_field(nx, ny, seed=7))
+    plan = _plan(torch, nx, ny, H, form)
+    dt = 10.0 / plan.rho
+    got = plan.grad_depth(x, G, dt).cpu().numpy()
+    ref = _plan(torch, nx, ny, H, "fp64", rtol=9e-14).grad_depth(x, G, dt).cpu().numpy()
+    assert rel_l2(got, ref) < 1e-9
+
+
+@pytest.mark.parametrize("form", ["fp64", "mixed"])
 def test_options_and_calls_left_to_the_lanczos_form(form):
     """A spacing h whose alias the expansion would have to resolve, and values
     outside the exponents that the expansion takes; and a rho set above the
