@@ -249,7 +249,9 @@ rexi_status rexi_plan_set_krylov(rexi_plan_t plan, double rtol, int32_t max_iter
  * plans):
  * REXI_KRYLOV_CG (default): one pole-pair CG solve per REXII term, terms
  *   batched (pair operator (alpha_{-n} - dt A)(alpha_n + dt A), Section 3's
- *   reduced sum); computes in the plan's form.
+ *   reduced sum); computes in the plan's form.  FP64 form: the reported
+ *   residual is an FP64 one of the FP64 system; the iterations before it run in
+ *   double-float where kappa 2^-46 <= rtol / 4, in FP64 otherwise.
  * REXI_KRYLOV_SHARED: one basis of the Krylov space of K = -i dt A
  *   (self-adjoint in the energy inner product) shared by every single-shift
  *   pole z_j of the step: (dt A - z_j)^{-1} f = -i (K + i z_j)^{-1} f, and the

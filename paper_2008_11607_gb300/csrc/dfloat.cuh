@@ -90,4 +90,22 @@ __device__ __forceinline__ double widen_float(float f) {
 // (hi, lo) -> double: one FP64 addition.
 __device__ __forceinline__ double df_to_double(float2 a) { return widen_float(a.x) + widen_float(a.y); }
 
+// The same operations for FP64 and double-float.
+// Sums of double-floats stay unnormalised inside a point's update (TwoSum of
+// the high parts, low parts added in FP32); one FastTwoSum at its end.
+__device__ __forceinline__ float2 u_add(float2 a, float2 b) {
+  const float s = a.x + b.x, bb = s - a.x;
+  return make_float2(s, ((a.x - (s - bb)) + (b.x - bb)) + (a.y + b.y));
+}
+__device__ __forceinline__ double u_add(double a, double b) { return a + b; }
+__device__ __forceinline__ float2 u_sub(float2 a, float2 b) { return u_add(a, make_float2(-b.x, -b.y)); }
+__device__ __forceinline__ double u_sub(double a, double b) { return a - b; }
+// acc + x c
+__device__ __forceinline__ float2 u_madd(float2 acc, float2 x, float2 c) {
+  return u_add(acc, f_mul(x.x, x.y, c.x, c.y));
+}
+__device__ __forceinline__ double u_madd(double acc, double x, double c) { return fma(x, c, acc); }
+__device__ __forceinline__ float2 u_norm(float2 a) { return f_fast(a.x, a.y); }
+__device__ __forceinline__ double u_norm(double a) { return a; }
+
 }  // namespace rexi
