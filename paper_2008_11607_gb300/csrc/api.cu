@@ -344,6 +344,10 @@ rexi_status rexi_plan_create(rexi_plan_t* out, int32_t nx, int32_t ny, double Lx
       p->fxh.twf = p->twf_xh;
       p->r2c = true;
     }
+    if (nx % 2 == 1) {  // odd: pairs of rows through the full-length plan
+      p->fxh = p->fx;
+      p->r2c = true;
+    }
     // rho(A): largest omega over the discrete wavenumbers (exact for constant depth)
     std::vector<double> sx2(nx), cx2(nx);
     for (int k = 0; k < nx; ++k) { sx2[k] = hx[k].y * hx[k].y; cx2[k] = hx[k].x * hx[k].x; }

@@ -77,9 +77,10 @@ cudaError_t fft2d_df(const double2* in, double2* out, int nfields, const FftPlan
 void split_twiddles(const double2* tw, int n, float4* out);  // host: FP64 table -> double-float
 // host: the double-float twiddle table of a transform (2 p.n entries: w[t], then grouped per stage)
 void df_twiddles(const double2* tw, const FftPlan1D& p, float4* out);
-// Real input (nx = 2 m even): forward transform of the real parts of `in`
-// into the half spectrum, ny x (m + 1) complex128 per field (field stride
-// ny (m + 1)), through an m-point transform per row (pxh: plan of length m);
+// Real input: forward transform of the real parts of `in` into the half
+// spectrum, ny x (nx/2 + 1) complex128 per field (field stride ny (nx/2 + 1)),
+// through an m-point transform per row (nx = 2 m even; pxh: plan of length m) or
+// an nx-point one per pair of rows (nx odd; pxh unused but for its tables);
 // inverse from the half spectrum (overwritten) to real fields (imaginary 0),
 // scaled.  df: 0 FP64; 1 double-float arithmetic (when every plan carries
 // double-float twiddles) with an FP64 half spectrum; 2 the same with the half
