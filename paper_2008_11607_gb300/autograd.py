@@ -1,6 +1,6 @@
 """torch.autograd bindings of the REXII step: gradients with respect to the
 state (the adjoint step, rexi_step_adjoint) and to the depth field
-(rexi_step_grad_depth), and a multi-step rollout that stores only every
+(rexi_step_grad_depth, both: rexi_step_backward), and a multi-step rollout that stores only every
 `every`-th state and recomputes the others during the backward pass.
 
 Argument marshalling only: the forward, adjoint and depth-gradient work all
@@ -27,9 +27,13 @@ class RexiStep(torch.autograd.Function):
         (state,) = ctx.saved_tensors
         plan, dt, tol, real = ctx.plan, ctx.dt, ctx.tol, ctx.real_input
         g = grad_out.contiguous()
-        grad_state = plan.step_adjoint(g, dt, tol=tol, real_input=real) if ctx.needs_input_grad[0] else None
-        grad_depth = None
-        if ctx.has_depth and ctx.needs_input_grad[1]:
+        grad_state = grad_depth = None
+        want_depth = ctx.has_depth and ctx.needs_input_grad[1]
+        if ctx.needs_input_grad[0] and want_depth:
+            grad_state, grad_depth = plan.step_backward(state.contiguous(), g, dt, tol=tol, real_input=real)
+        elif ctx.needs_input_grad[0]:
+            grad_state = plan.step_adjoint(g, dt, tol=tol, real_input=real)
+        elif want_depth:
             grad_depth = plan.grad_depth(state.contiguous(), g, dt, tol=tol, real_input=real)
         return grad_state, grad_depth, None, None, None, None
 
@@ -65,7 +69,6 @@ class RexiRollout(torch.autograd.Function):
         grad_depth = None
         if want_depth:
             grad_depth = torch.zeros((plan.ny, plan.nx), dtype=torch.float64, device=g.device)
-        ws = None
         for seg in reversed(range(len(ckpts))):
             first = seg * ctx.every
             last = min(first + ctx.every, ctx.nsteps)
@@ -74,8 +77,9 @@ class RexiRollout(torch.autograd.Function):
                 states.append(plan.step(states[-1], dt, tol=tol, real_input=real))
             for j in reversed(range(last - first)):
                 if want_depth:
-                    plan.grad_depth(states[j], g, dt, tol=tol, real_input=real, grad=grad_depth, workspace=ws)
-                g = plan.step_adjoint(g, dt, tol=tol, real_input=real)
+                    g, _ = plan.step_backward(states[j], g, dt, tol=tol, real_input=real, grad=grad_depth)
+                else:
+                    g = plan.step_adjoint(g, dt, tol=tol, real_input=real)
         return g, grad_depth, None, None, None, None, None, None
 
 

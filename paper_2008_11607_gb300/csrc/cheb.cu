@@ -971,7 +971,7 @@ rexi_status step_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
 
 template <typename T>
 rexi_status grad_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, const void* f_in, const void* g_out,
-                      double* grad_depth, double dt, const ChebGradBuffers& b, cudaStream_t s,
+                      double* grad_depth, void* grad_in, double dt, const ChebGradBuffers& b, cudaStream_t s,
                       const KrylovHooks& hooks, double* bound) {
   auto mark = [&](int i) {
     if (hooks.mark) hooks.mark(hooks.ctx, i, s);
@@ -1070,6 +1070,8 @@ rexi_status grad_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
     A.s = sf;
     A.grad = grad_depth;
     A.w = k->w64;
+    A.out = static_cast<double2*>(grad_in);
+    A.adjoint = A.real_out = 1;
     launch_step<T, kGradLast>(G, A, 1, s, !many);
     ++launches;
   }
@@ -1127,11 +1129,11 @@ rexi_status cheb_step(KrylovSettings* k, const ChebPlan& p, int df, double h, in
 }
 
 rexi_status cheb_grad(KrylovSettings* k, const ChebPlan& p, int df, double h, int M, const void* f_in,
-                      const void* g_out, double* grad_depth, double dt, const ChebGradBuffers& b, cudaStream_t s,
-                      const KrylovHooks& hooks, double* bound) {
+                      const void* g_out, double* grad_depth, void* grad_in, double dt, const ChebGradBuffers& b,
+                      cudaStream_t s, const KrylovHooks& hooks, double* bound) {
   *bound = 0.0;
-  return df ? grad_impl<float2>(k, p, h, M, f_in, g_out, grad_depth, dt, b, s, hooks, bound)
-            : grad_impl<double>(k, p, h, M, f_in, g_out, grad_depth, dt, b, s, hooks, bound);
+  return df ? grad_impl<float2>(k, p, h, M, f_in, g_out, grad_depth, grad_in, dt, b, s, hooks, bound)
+            : grad_impl<double>(k, p, h, M, f_in, g_out, grad_depth, grad_in, dt, b, s, hooks, bound);
 }
 
 }  // namespace rexi

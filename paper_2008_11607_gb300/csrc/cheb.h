@@ -43,10 +43,11 @@ struct ChebGradBuffers {
   void* exchange;      // edge values between warps (any size; 256-byte aligned)
   size_t exchange_bytes;
 };
-// grad_depth += dL/dH for out = r(dt A(H)) f_in, G = dL/d out (real input);
-// same refusals, with grad_depth untouched.
+// grad_depth += dL/dH for out = r(dt A(H)) f_in, G = dL/d out (real input), and,
+// with grad_in, grad_in = r(dt A)^H G: the end of the same recurrence.  Same
+// refusals, with both untouched.
 rexi_status cheb_grad(KrylovSettings* k, const ChebPlan& p, int df, double h, int M, const void* f_in,
-                      const void* g_out, double* grad_depth, double dt, const ChebGradBuffers& b, cudaStream_t s,
-                      const KrylovHooks& hooks, double* bound);
+                      const void* g_out, double* grad_depth, void* grad_in, double dt, const ChebGradBuffers& b,
+                      cudaStream_t s, const KrylovHooks& hooks, double* bound);
 
 }  // namespace rexi

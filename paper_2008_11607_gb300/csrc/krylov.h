@@ -54,14 +54,16 @@ rexi_status lanczos_tables(KrylovSettings* k);  // fills Hdf, wdf
 size_t lanczos_grad_workspace_bytes(const KrylovSettings* k, int M, double h);
 rexi_status krylov_grad_depth_lanczos(KrylovSettings* k, int form, double h, int M, const void* f_in,
                                       const void* g_out,
-                                      double* grad_depth, double dt, void* ws, size_t ws_bytes, cudaStream_t s,
-                                      rexi_step_info* info, const KrylovHooks& hooks);
+                                      double* grad_depth, void* grad_in, double dt, void* ws, size_t ws_bytes,
+                                      cudaStream_t s, rexi_step_info* info, const KrylovHooks& hooks,
+                                      bool* grad_in_done);
 rexi_status krylov_step_lanczos(KrylovSettings* k, int form, double h, int M, const void* in, void* out, double dt,
                                 int real_input, int term_begin, int term_end, void* ws, size_t ws_bytes,
                                 cudaStream_t s, rexi_step_info* info, bool adjoint, const KrylovHooks& hooks);
-// grad_depth += dL/dH for out = r(dt A(H)) f_in and G = dL/d out.
+// grad_depth += dL/dH for out = r(dt A(H)) f_in and G = dL/d out.  grad_in
+// (nullable): r(dt A)^H G as well where that comes with it (*grad_in_done).
 rexi_status krylov_grad_depth(KrylovSettings* k, int form, double h, int M, const void* f_in, const void* g_out,
-                              double* grad_depth, double dt, int real_input, void* ws, size_t ws_bytes,
-                              cudaStream_t s, rexi_step_info* info, const KrylovHooks& hooks);
+                              double* grad_depth, void* grad_in, double dt, int real_input, void* ws, size_t ws_bytes,
+                              cudaStream_t s, rexi_step_info* info, const KrylovHooks& hooks, bool* grad_in_done);
 
 }  // namespace rexi

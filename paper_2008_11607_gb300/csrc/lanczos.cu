@@ -1619,8 +1619,9 @@ size_t lanczos_grad_workspace_bytes(const KrylovSettings* k, int M, double h) { 
 
 rexi_status krylov_grad_depth_lanczos(KrylovSettings* k, int form, double h, int M, const void* f_in,
                                       const void* g_out,
-                                      double* grad_depth, double dt, void* ws, size_t ws_bytes, cudaStream_t s,
-                                      rexi_step_info* info, const KrylovHooks& hooks) {
+                                      double* grad_depth, void* grad_in, double dt, void* ws, size_t ws_bytes,
+                                      cudaStream_t s, rexi_step_info* info, const KrylovHooks& hooks,
+                                      bool* grad_in_done) {
   using cd = std::complex<double>;
   auto mark = [&](int i) {
     if (hooks.mark) hooks.mark(hooks.ctx, i, s);
@@ -1645,7 +1646,9 @@ rexi_status krylov_grad_depth_lanczos(KrylovSettings* k, int form, double h, int
                                 b + L.basB, b + L.part, b + L.basA + 2 * L.vb, (size_t)(L.cap - 2) * L.vb};
     double tail = 0.0;
     const rexi_status st =
-        cheb_grad(k, cp, form == REXI_FORM_MIXED ? 1 : 0, h, M, f_in, g_out, grad_depth, dt, cb, s, hooks, &tail);
+        cheb_grad(k, cp, form == REXI_FORM_MIXED ? 1 : 0, h, M, f_in, g_out, grad_depth, grad_in, dt, cb, s, hooks,
+                  &tail);
+    if (st == REXI_OK) *grad_in_done = grad_in != nullptr;
     if (st == REXI_OK && info) {
       memset(info, 0, sizeof(*info));
       info->N = N;

@@ -90,6 +90,7 @@ SIGNATURES = {
     "rexi_step": (_c_int, [_vp, _vp, _vp, _c_dbl, _c_dbl, _c_int, _c_int, _c_int, _vp, ctypes.c_size_t, _vp,
                            ctypes.POINTER(rexi_step_info)]),
     "rexi_step_adjoint": (_c_int, [_vp, _vp, _vp, _c_dbl, _c_dbl, _c_int, _vp, ctypes.c_size_t, _vp]),
+    "rexi_step_backward": (_c_int, [_vp, _vp, _vp, _vp, _vp, _c_dbl, _c_dbl, _c_int, _vp, ctypes.c_size_t, _vp]),
     "rexi_step_grad_depth": (_c_int, [_vp, _vp, _vp, _vp, _c_dbl, _c_dbl, _c_int, _vp, ctypes.c_size_t, _vp,
                                       ctypes.POINTER(rexi_step_info)]),
     "rexi_step_host_async": (_c_int, [_vp, _vp, _vp, _c_dbl, _c_dbl, _c_int, _vp, ctypes.c_size_t, _vp]),
@@ -410,6 +411,21 @@ class Plan:
                                             _stream_handle(stream), ctypes.byref(info) if info is not None else None)
         _check(st, "rexi_step_grad_depth")
         return (grad, info) if want_info else grad
+
+    def step_backward(self, state, grad_out, dt, tol=1e-10, real_input=True, grad=None, workspace=None, stream=None):
+        """(grad_state, grad): the adjoint step and grad += dL/dH in one call (variable depth)."""
+        import torch
+
+        if grad is None:
+            grad = torch.zeros((self.ny, self.nx), dtype=torch.float64, device=state.device)
+        if workspace is None:
+            n = max(self.workspace_size(dt, tol, real_input), self.workspace_size(dt, tol, real_input, grad_depth=True))
+            workspace = torch.empty(n, dtype=torch.uint8, device=state.device)
+        out = torch.empty_like(grad_out)
+        st = self._lib.rexi_step_backward(self._h, _ptr(state), _ptr(grad_out), _ptr(out), _ptr(grad), dt, tol,
+                                          int(real_input), _ptr(workspace), workspace.numel(), _stream_handle(stream))
+        _check(st, "rexi_step_backward")
+        return out, grad
 
     def step_adjoint(self, grad_out, dt, tol=1e-10, real_input=True, out=None, workspace=None, stream=None):
         import torch
