@@ -234,8 +234,8 @@ __global__ void __launch_bounds__(256) batch_combine_kernel(double2* spec, const
   OrbitScalars o;
   if (!(half && df)) o = orb[D.orb_off + at];
   if (!half) {
-    combine_scaled(spec + D.spec_off, (size_t)k, (size_t)nk, symbol_entries(sp, kx, ky, adjoint != 0),
-                   make_double2(D.R0re, D.R0im), o, adjoint != 0);
+    combine_staggered(spec + D.spec_off, (size_t)k, (size_t)nk, sp, kx, ky, make_double2(D.R0re, D.R0im), o,
+                      adjoint != 0);
   } else if (df) {
     const OrbitScalarsDF od = reinterpret_cast<const OrbitScalarsDF*>(orb + D.orb_off)[at];
     SymbolDF sd;
@@ -250,8 +250,8 @@ __global__ void __launch_bounds__(256) batch_combine_kernel(double2* spec, const
                   df_from_double(D.R0re), od.s1, od.s2, adjoint != 0);
   } else {
     o.s2im = 0.0;
-    combine_scaled(spec + D.half_off, (size_t)k, (size_t)nk, symbol_entries(sp, kx, ky, adjoint != 0),
-                   make_double2(D.R0re, 0.0), o, adjoint != 0);
+    combine_staggered(spec + D.half_off, (size_t)k, (size_t)nk, sp, kx, ky, make_double2(D.R0re, 0.0), o,
+                      adjoint != 0);
   }
 }
 

@@ -231,6 +231,54 @@ __device__ __forceinline__ void combine_scaled(double2* spec, size_t idx, size_t
   }
 }
 
+// The same on the C grid with the staggering rotated out.  With u = e^{i a} U,
+// v = e^{i b} V (a, b the half angles), ax = 2 sin(a) / dx, ay = 2 sin(b) / dy and
+// F = f cos(a) cos(b),
+//   (B f)_eta = -i H (ax U + ay V),  (B f)_U = -i g ax eta + F V,  (B f)_V = -i g ay eta - F U:
+// every product with a complex value is one with a real or imaginary number (12
+// FP64 operations per application instead of 24, 16 for the two rotations and
+// back); B^H has -g, -H, -f in the places of H, g, f.  Bound by the FP64 pipe
+// (double-float form: by FP32 issue): 2048^2 step, FP64 2575 -> 2431 us, mixed 835 -> 814.
+__device__ __forceinline__ void combine_staggered(double2* spec, size_t idx, size_t fs, const SymbolParams& sp, int kx,
+                                                  int ky, double2 c0, OrbitScalars o, bool adjoint) {
+  const double2 hx = sp.half_x[kx], hy = sp.half_y[ky];
+  const double ax = 2.0 * hx.y * sp.inv_dx, ay = 2.0 * hy.y * sp.inv_dy;
+  const double p = adjoint ? -sp.g : sp.H, q = adjoint ? -sp.H : sp.g;
+  const double px = p * ax, py = p * ay, qx = q * ax, qy = q * ay;
+  const double F = (adjoint ? -sp.f : sp.f) * (hx.x * hy.x);
+  const double2 u = spec[idx + fs], v = spec[idx + 2 * fs];
+  const double2 f0 = spec[idx], f1 = cm(cj(hx), u), f2 = cm(cj(hy), v);
+  auto apply = [&](double2 a, double2 b, double2 c, double2 y[3]) {
+    y[0] = make_double2(fma(px, b.y, py * c.y), -fma(px, b.x, py * c.x));
+    y[1] = make_double2(fma(qx, a.y, F * c.x), fma(-qx, a.x, F * c.y));
+    y[2] = make_double2(fma(qy, a.y, -F * b.x), -fma(qy, a.x, F * b.y));
+  };
+  double2 y1[3], y2[3], out[3];
+  apply(f0, f1, f2, y1);
+  apply(y1[0], y1[1], y1[2], y2);
+  const double2 f[3] = {f0, f1, f2};
+  if (c0.y == 0.0 && o.s2im == 0.0) {  // real input
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      out[c] = make_double2(fma(o.s2re, y2[c].x, fma(o.s1, y1[c].x, c0.x * f[c].x)),
+                            fma(o.s2re, y2[c].y, fma(o.s1, y1[c].y, c0.x * f[c].y)));
+  } else {
+    double2 s2 = make_double2(o.s2re, o.s2im);
+    if (adjoint) {
+      c0 = cj(c0);
+      s2 = cj(s2);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double2 t = cm(c0, f[c]);
+      out[c] = cma(s2, y2[c], make_double2(fma(o.s1, y1[c].x, t.x), fma(o.s1, y1[c].y, t.y)));
+    }
+  }
+  spec[idx] = out[0];
+  spec[idx + fs] = cm(hx, out[1]);
+  spec[idx + 2 * fs] = cm(hy, out[2]);
+}
+
 // Double-float combine on a double-float half spectrum (real input, C-grid):
 // out = c0 f + s1 B f + s2 B^2 f with real c0 = Re R0, s1, s2; the symbol from
 // double-float half-angle tables (cos, sin of pi k / n as float4 hi/lo pairs).
@@ -243,35 +291,37 @@ struct SymbolDF {
 __device__ __forceinline__ float4 c_of(float2 re, float2 im) { return make_float4(re.x, re.y, im.x, im.y); }
 __device__ __forceinline__ float2 f_neg(float2 a) { return make_float2(-a.x, -a.y); }
 
-// The six non-zero entries of the C-grid symbol at (kx, ky) in double-float
-// (B^H for the adjoint): e[0..5] = B01, B02, B10, B12, B20, B21.
-__device__ __forceinline__ void symbol_df(const SymbolDF& sd, int kx, int ky, bool adjoint, float4 e[6]) {
-  const float4 hx = sd.half_x[kx], hy = sd.half_y[ky];
-  const float2 cx = make_float2(hx.x, hx.y), sx = make_float2(hx.z, hx.w);
-  const float2 cy = make_float2(hy.x, hy.y), sy = make_float2(hy.z, hy.w);
-  const float2 ax = f_mulf(make_float2(2.f * sx.x, 2.f * sx.y), sd.inv_dx);
-  const float2 ay = f_mulf(make_float2(2.f * sy.x, 2.f * sy.y), sd.inv_dy);
-  const float2 Hax = f_neg(f_mulf(sd.H, ax)), Hay = f_neg(f_mulf(sd.H, ay));
-  const float2 gax = f_mulf(sd.g, ax), gay = f_mulf(sd.g, ay);
-  e[0] = c_of(f_mulf(Hax, sx), f_mulf(Hax, cx));        // -H dxb
-  e[1] = c_of(f_mulf(Hay, sy), f_mulf(Hay, cy));        // -H dyb
-  e[2] = c_of(f_mulf(gax, sx), f_neg(f_mulf(gax, cx)));  // -g dxf
-  e[4] = c_of(f_mulf(gay, sy), f_neg(f_mulf(gay, cy)));  // -g dyf
-  const float2 cxcy = f_mulf(cx, cy);
-  const float2 fcc = f_mulf(sd.f, cxcy);
-  const float2 pr = f_mulf(fcc, f_addf(cxcy, f_mulf(sx, sy)));
-  const float2 pim = f_mulf(fcc, f_subf(f_mulf(sx, cy), f_mulf(cx, sy)));
-  e[3] = c_of(pr, pim);          // f P
-  e[5] = c_of(f_neg(pr), pim);   // -f conj(P)
-  if (adjoint) {  // (B^H)_ij = conj(B_ji)
-    const float4 t01 = e[0], t02 = e[1], t10 = e[2], t12 = e[3], t20 = e[4], t21 = e[5];
-    e[0] = cconj(t10);
-    e[1] = cconj(t20);
-    e[2] = cconj(t01);
-    e[3] = cconj(t21);
-    e[4] = cconj(t02);
-    e[5] = cconj(t12);
-  }
+// B f and B^2 f in the rotated unknowns of combine_staggered, in double-float.
+struct StaggeredDF {
+  float4 ex, ey;  // e^{i a}, e^{i b}
+  float2 px, py, qx, qy, F;
+};
+__device__ __forceinline__ StaggeredDF staggered_df(const SymbolDF& sd, int kx, int ky, bool adjoint) {
+  StaggeredDF S;
+  S.ex = sd.half_x[kx];
+  S.ey = sd.half_y[ky];
+  const float2 ax = f_mulf(make_float2(2.f * S.ex.z, 2.f * S.ex.w), sd.inv_dx);
+  const float2 ay = f_mulf(make_float2(2.f * S.ey.z, 2.f * S.ey.w), sd.inv_dy);
+  const float2 p = adjoint ? f_neg(sd.g) : sd.H, q = adjoint ? f_neg(sd.H) : sd.g;
+  S.px = f_mulf(p, ax);
+  S.py = f_mulf(p, ay);
+  S.qx = f_mulf(q, ax);
+  S.qy = f_mulf(q, ay);
+  S.F = f_mulf(adjoint ? f_neg(sd.f) : sd.f, f_mulf(make_float2(S.ex.x, S.ex.y), make_float2(S.ey.x, S.ey.y)));
+  return S;
+}
+// a x + b y for double-floats
+__device__ __forceinline__ float2 f_dot2(float2 a, float2 x, float2 b, float2 y) {
+  const float2 s = f_mul(a.x, a.y, x.x, x.y), t = f_mul(b.x, b.y, y.x, y.y);
+  return f_add(s.x, s.y, t.x, t.y);
+}
+__device__ __forceinline__ void apply_staggered(const StaggeredDF& S, const float4 f[3], float4 y[3]) {
+  const float2 ar = make_float2(f[0].x, f[0].y), ai = make_float2(f[0].z, f[0].w);
+  const float2 br = make_float2(f[1].x, f[1].y), bi = make_float2(f[1].z, f[1].w);
+  const float2 cr_ = make_float2(f[2].x, f[2].y), ci = make_float2(f[2].z, f[2].w);
+  y[0] = c_of(f_dot2(S.px, bi, S.py, ci), f_neg(f_dot2(S.px, br, S.py, cr_)));
+  y[1] = c_of(f_dot2(S.qx, ai, S.F, cr_), f_dot2(f_neg(S.qx), ar, S.F, ci));
+  y[2] = c_of(f_dot2(S.qy, ai, f_neg(S.F), br), f_neg(f_dot2(S.qy, ar, S.F, bi)));
 }
 
 // Complex input on an FP64 spectrum: values become double-float pairs on load
@@ -279,23 +329,21 @@ __device__ __forceinline__ void symbol_df(const SymbolDF& sd, int kx, int ky, bo
 // complex (r(0) enters whole), s1 real.
 __device__ __forceinline__ void combine_dfc_at(double2* spec, size_t k, size_t nk, int kx, int ky, const SymbolDF& sd,
                                                float4 c0, float2 s1, float4 s2, bool adjoint) {
-  float4 e[6];
-  symbol_df(sd, kx, ky, adjoint, e);
+  const StaggeredDF S = staggered_df(sd, kx, ky, adjoint);
   float4 f[3], y1[3], y2[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const double2 v = spec[k + c * nk];
     f[c] = c_of(df_from_double(v.x), df_from_double(v.y));
   }
-  y1[0] = cadd(cmul(e[0], f[1]), cmul(e[1], f[2]));
-  y1[1] = cadd(cmul(e[2], f[0]), cmul(e[3], f[2]));
-  y1[2] = cadd(cmul(e[4], f[0]), cmul(e[5], f[1]));
-  y2[0] = cadd(cmul(e[0], y1[1]), cmul(e[1], y1[2]));
-  y2[1] = cadd(cmul(e[2], y1[0]), cmul(e[3], y1[2]));
-  y2[2] = cadd(cmul(e[4], y1[0]), cmul(e[5], y1[1]));
+  f[1] = cmul(cconj(S.ex), f[1]);
+  f[2] = cmul(cconj(S.ey), f[2]);
+  apply_staggered(S, f, y1);
+  apply_staggered(S, y1, y2);
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const float4 o = cadd(cadd(cmul(c0, f[c]), crmul(s1, y1[c])), cmul(s2, y2[c]));
+    float4 o = cadd(cadd(cmul(c0, f[c]), crmul(s1, y1[c])), cmul(s2, y2[c]));
+    if (c) o = cmul(c == 1 ? S.ex : S.ey, o);
     spec[k + c * nk] = make_double2(df_to_double(make_float2(o.x, o.y)), df_to_double(make_float2(o.z, o.w)));
   }
 }
@@ -303,45 +351,20 @@ __device__ __forceinline__ void combine_dfc_at(double2* spec, size_t k, size_t n
 // In place at index k of the three fields (field stride nk), wavenumber (kx, ky).
 __device__ __forceinline__ void combine_df_at(float4* spec, size_t k, size_t nk, int kx, int ky, const SymbolDF& sd,
                                               float2 c0, float2 s1, float2 s2, bool adjoint) {
-  const float4 hx = sd.half_x[kx], hy = sd.half_y[ky];
-  const float2 cx = make_float2(hx.x, hx.y), sx = make_float2(hx.z, hx.w);
-  const float2 cy = make_float2(hy.x, hy.y), sy = make_float2(hy.z, hy.w);
-  // a = 2 sin(theta/2) / dx; B entries with g, H, f folded in (see symbol_at)
-  const float2 ax = f_mulf(make_float2(2.f * sx.x, 2.f * sx.y), sd.inv_dx);
-  const float2 ay = f_mulf(make_float2(2.f * sy.x, 2.f * sy.y), sd.inv_dy);
-  const float2 Hax = f_neg(f_mulf(sd.H, ax)), Hay = f_neg(f_mulf(sd.H, ay));
-  const float2 gax = f_mulf(sd.g, ax), gay = f_mulf(sd.g, ay);
-  float4 e01 = c_of(f_mulf(Hax, sx), f_mulf(Hax, cx));        // -H dxb
-  float4 e02 = c_of(f_mulf(Hay, sy), f_mulf(Hay, cy));        // -H dyb
-  float4 e10 = c_of(f_mulf(gax, sx), f_neg(f_mulf(gax, cx)));  // -g dxf
-  float4 e20 = c_of(f_mulf(gay, sy), f_neg(f_mulf(gay, cy)));  // -g dyf
-  const float2 cxcy = f_mulf(cx, cy);
-  const float2 fcc = f_mulf(sd.f, cxcy);
-  const float2 pr = f_mulf(fcc, f_addf(cxcy, f_mulf(sx, sy)));
-  const float2 pim = f_mulf(fcc, f_subf(f_mulf(sx, cy), f_mulf(cx, sy)));
-  float4 e12 = c_of(pr, pim);          // f P
-  float4 e21 = c_of(f_neg(pr), pim);   // -f conj(P)
-  if (adjoint) {  // B^H: (B^H)_ij = conj(B_ji)
-    const float4 t01 = e01, t02 = e02, t10 = e10, t12 = e12, t20 = e20, t21 = e21;
-    e01 = cconj(t10);
-    e02 = cconj(t20);
-    e10 = cconj(t01);
-    e12 = cconj(t21);
-    e20 = cconj(t02);
-    e21 = cconj(t12);
-  }
+  const StaggeredDF S = staggered_df(sd, kx, ky, adjoint);
   float4 f[3], y1[3], y2[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) f[c] = spec[k + c * nk];
-  y1[0] = cadd(cmul(e01, f[1]), cmul(e02, f[2]));
-  y1[1] = cadd(cmul(e10, f[0]), cmul(e12, f[2]));
-  y1[2] = cadd(cmul(e20, f[0]), cmul(e21, f[1]));
-  y2[0] = cadd(cmul(e01, y1[1]), cmul(e02, y1[2]));
-  y2[1] = cadd(cmul(e10, y1[0]), cmul(e12, y1[2]));
-  y2[2] = cadd(cmul(e20, y1[0]), cmul(e21, y1[1]));
+  f[1] = cmul(cconj(S.ex), f[1]);
+  f[2] = cmul(cconj(S.ey), f[2]);
+  apply_staggered(S, f, y1);
+  apply_staggered(S, y1, y2);
 #pragma unroll
-  for (int c = 0; c < 3; ++c)
-    spec[k + c * nk] = cadd(cadd(crmul(c0, f[c]), crmul(s1, y1[c])), crmul(s2, y2[c]));
+  for (int c = 0; c < 3; ++c) {
+    float4 o = cadd(cadd(crmul(c0, f[c]), crmul(s1, y1[c])), crmul(s2, y2[c]));
+    if (c) o = cmul(c == 1 ? S.ex : S.ey, o);
+    spec[k + c * nk] = o;
+  }
 }
 
 // Map thread -> wavenumber pair.  Pairs (k, -k) with ky in [0, ny/2]; in the

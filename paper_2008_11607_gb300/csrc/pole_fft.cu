@@ -207,7 +207,10 @@ __global__ void __launch_bounds__(256) pole_orbit_combine_kernel(double2* spec,
   if (k >= nk) return;
   const int ky = (int)(k / row_len), kx = (int)(k - (size_t)ky * row_len);
   const OrbitScalars o = fin[orbit_of(op, sp.nx, sp.ny, kx, ky)];
-  combine_scaled(spec, k, nk, symbol_entries(sp, kx, ky, adjoint != 0), R0, o, adjoint != 0);
+  if (sp.spectral)
+    combine_scaled(spec, k, nk, symbol_entries(sp, kx, ky, adjoint != 0), R0, o, adjoint != 0);
+  else
+    combine_staggered(spec, k, nk, sp, kx, ky, R0, o, adjoint != 0);
 }
 
 // Double-float combine on a double-float half spectrum (see combine_df_at).
