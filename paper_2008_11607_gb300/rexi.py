@@ -245,6 +245,13 @@ def alu_probe(kind, blocks, iters, out, stream=None):
     return blocks * 256 * 256 * iters * 2 * (2 if k == 2 else 1)
 
 
+def _own(t, stream):
+    """A tensor allocated here for a call on `stream`: its memory is not reused before that stream is done."""
+    if stream is not None:
+        t.record_stream(stream)
+    return t
+
+
 class Plan:
     """Owns one rexi_plan_t.  ``depth`` (torch float64 CUDA tensor, (ny, nx))
     selects the variable-depth path; it must stay alive as long as the plan."""
@@ -346,9 +353,9 @@ class Plan:
         import torch
 
         if out is None:
-            out = torch.empty_like(state)
+            out = _own(torch.empty_like(state), stream)
         if workspace is None:
-            workspace = self.workspace(dt, tol, real_input, device=state.device)
+            workspace = _own(self.workspace(dt, tol, real_input, device=state.device), stream)
         info = rexi_step_info() if want_info else None
         st = self._lib.rexi_step(self._h, _ptr(state), _ptr(out), dt, tol, int(real_input), int(terms[0]),
                                  int(terms[1]), _ptr(workspace), workspace.numel(), _stream_handle(stream),
@@ -404,7 +411,7 @@ class Plan:
         if grad is None:
             grad = torch.zeros((self.ny, self.nx), dtype=torch.float64, device=state.device)
         if workspace is None:
-            workspace = self.workspace(dt, tol, real_input, device=state.device, grad_depth=True)
+            workspace = _own(self.workspace(dt, tol, real_input, device=state.device, grad_depth=True), stream)
         info = rexi_step_info() if want_info else None
         st = self._lib.rexi_step_grad_depth(self._h, _ptr(state), _ptr(grad_out), _ptr(grad), dt, tol,
                                             int(real_input), _ptr(workspace), workspace.numel(),
@@ -420,8 +427,8 @@ class Plan:
             grad = torch.zeros((self.ny, self.nx), dtype=torch.float64, device=state.device)
         if workspace is None:
             n = max(self.workspace_size(dt, tol, real_input), self.workspace_size(dt, tol, real_input, grad_depth=True))
-            workspace = torch.empty(n, dtype=torch.uint8, device=state.device)
-        out = torch.empty_like(grad_out)
+            workspace = _own(torch.empty(n, dtype=torch.uint8, device=state.device), stream)
+        out = _own(torch.empty_like(grad_out), stream)
         st = self._lib.rexi_step_backward(self._h, _ptr(state), _ptr(grad_out), _ptr(out), _ptr(grad), dt, tol,
                                           int(real_input), _ptr(workspace), workspace.numel(), _stream_handle(stream))
         _check(st, "rexi_step_backward")
@@ -431,9 +438,9 @@ class Plan:
         import torch
 
         if out is None:
-            out = torch.empty_like(grad_out)
+            out = _own(torch.empty_like(grad_out), stream)
         if workspace is None:
-            workspace = self.workspace(dt, tol, real_input, device=grad_out.device)
+            workspace = _own(self.workspace(dt, tol, real_input, device=grad_out.device), stream)
         st = self._lib.rexi_step_adjoint(self._h, _ptr(grad_out), _ptr(out), dt, tol, int(real_input),
                                          _ptr(workspace), workspace.numel(), _stream_handle(stream))
         _check(st, "rexi_step_adjoint")
