@@ -42,41 +42,13 @@ N_SEEDS = 10
 METRIC = "grid-points×poles solved/sec and HBM GB/s vs roofline at stated error vs FP64 oracle"
 UNIT = "grid-points*poles/s"
 
-# Per-term work of the pole-sum loops, counted from the kernel source
-# (csrc/pole_common.cuh).  mixed (h n on the split grid, as at h = 0.5): 62
-# FP32 arithmetic instructions per term (14 of them FFMA) plus the
-# renormalisation of both accumulators every 16 terms (6 / 16) -> 62.375
-# operations, 76.375 flops; besides these, one FMNMX pair and the MUFU
-# reciprocal seed.  fp64: 8 DFMA + 1 DADD -> 17 flops, one MUFU
-# seed.  The sum runs once per orbit of omega's symmetries ((+-kx, +-ky) and
-# kx <-> ky on the square grid).
-FLOPS_PER_TERM = {"mixed": 76.375, "fp64": 17}
-FP32_INSTR_PER_TERM = 62.375
-FP64_INSTR_PER_TERM = 9
-# Peaks for ALU-bound kernels, derived from unit counts and the maximum clock:
-# 152 SMs x 128 FP32 lanes x 2 flops (FMA) x 2.07 GHz; FP64 from the nominal
-# 1.25 TFLOP/s of this GPU.
-SMS = 152
-SM_MAX_GHZ = 2.07
-PEAK_FP32_TFLOPS = SMS * 128 * 2 * SM_MAX_GHZ / 1e3
-PEAK_FP64_TFLOPS = 1.25
-# DRAM traffic per launch of the pole-sum kernel and of the combine pass from
-# ncu captures on the 2048^2 grid (the traffic does not depend on the term
-# count); None where no capture of the current kernel exists.
-NCU_POLE_TRAFFIC_BYTES = {"mixed": 283648 + 3840, "fp64": None}  # 2048^2, tau rho = 1000 (one-pass capture)
-# the combine pass of the mixed form at 2048^2 (pole_orbit_finalize_kernel +
-# pole_orbit_combine_df_kernel, one launch each, one-pass capture): DRAM bytes
-NCU_COMBINE_TRAFFIC_BYTES = (16884480 + 0) + (110867200 + 37490176)
+# DRAM traffic per launch from ncu captures on the 2048^2 grid:
+# the combine pass of the mixed form (pole_orbit_combine_df_kernel)
+NCU_COMBINE_TRAFFIC_BYTES = 110867200 + 37490176
 # the forward double-float transform of real input at 2048^2 (fft_rows_r2c_kernel
 # + fft_cols_kernel, one launch each; one-pass capture of the current
 # kernels): DRAM bytes read + written by the two launches
 NCU_FFT_FWD_TRAFFIC_BYTES = (201528832 + 66863616) + (100910080 + 42878720)
-
-
-def orbit_count(n):
-    """Orbits of the n x n wavenumber grid under omega's symmetries."""
-    a = n // 2 + 1
-    return a * (a + 1) // 2
 
 
 def set_workload(grid, tau_rho):
@@ -431,15 +403,14 @@ def krylov_measure(torch, rexi, inputs, form, n_terms, rtol, warm=1):
     }
 
 
-LANCZOS_BYTES_PER_PT_STEP = 88  # lz_wstep, first pass (real form): W_{j-1}, W_{j-2} (24 B each) + H, g/H (8 B
-# each) in; W_j (24 B) out
+CHEB_BYTES_PER_PT_STEP = 104  # cheb_step_kernel: b_{k+1}, b_{k+2}, F (24 B each) + H (8 B) read, b_k (24 B) written
 
 
 def shared_measure(torch, rexi, inputs, rtol=1e-10, reps=3, n=None, tau_rho=None, keep=True, form="mixed"):
     """Variable-depth workload, every REXII term (1024^2, tau rho = 400), by the
-    shared-Krylov method (one Lanczos basis for all poles; FP64, or
-    double-float vectors for the mixed form): with the minimum workspace
-    (second pass regenerates the basis) and with the basis kept in HBM."""
+    shared-Krylov method (one Chebyshev basis for all poles; FP64, or
+    double-float vectors for the mixed form), with the minimum workspace and, with
+    `keep`, with room for a basis (which the Chebyshev form does not use)."""
     import numpy as np
 
     n = n or KRYLOV_D
@@ -458,7 +429,7 @@ def shared_measure(torch, rexi, inputs, rtol=1e-10, reps=3, n=None, tau_rho=None
     _, info = plan.step(x, dt, out=out, want_info=True)
     kk = int(info.krylov_iters)
     res = {}
-    for label, extra in (("regenerate", 0), ("kept_basis", kk + 64))[:2 if keep else 1]:
+    for label, extra in (("minimum_workspace", 0), ("large_workspace", kk + 64))[:2 if keep else 1]:
         ws = torch.empty(base + extra * vec, dtype=torch.uint8, device="cuda")
         plan.step(x, dt, out=out, workspace=ws)
         torch.cuda.synchronize()
@@ -476,23 +447,21 @@ def shared_measure(torch, rexi, inputs, rtol=1e-10, reps=3, n=None, tau_rho=None
         J = int(info.n_poles)
         steps_run = int(info.krylov_term_iters)
         pass1 = ph[0] / max(ncalls, 1)
-        gbs = LANCZOS_BYTES_PER_PT_STEP * n * n * steps_run / (pass1 / 1e3) / 1e9
+        gbs = CHEB_BYTES_PER_PT_STEP * n * n * steps_run / (pass1 / 1e3) / 1e9
         o = out.cpu().numpy()
         en = lambda v: float(np.sqrt(np.sum(1.0 / Hn * np.abs(v[0]) ** 2) + np.sum(np.abs(v[1:]) ** 2)))
         res[label] = {
             "value": n * n * J / (ms / 1e3), "unit": UNIT, "ms_per_step": ms, "workspace_gb": ws.numel() / 1e9,
-            "lanczos_steps": int(info.krylov_iters), "first_pass_steps": steps_run,
+            "basis_steps": int(info.krylov_iters),
             "error_bound": info.krylov_max_rel_res,
-            "phases_ms": {"first_pass": pass1, "coefficients": ph[1] / max(ncalls, 1),
-                          "second_pass": ph[2] / max(ncalls, 1), "setup": ph[3] / max(ncalls, 1)},
+            "phases_ms": {"steps": pass1, "last_step": ph[2] / max(ncalls, 1), "setup": ph[3] / max(ncalls, 1)},
             "energy_drift": abs(en(o) / en(xn) - 1.0),
-            "roofline": {"kernel": "%s (first pass, incl. bound checks in the time)"
-                                   % ("lz_dfstep" if form == "mixed" else "lz_wstep"), "bound": "hbm",
-                         "achieved": gbs, "unit": "GB/s", "bytes_per_point_step": LANCZOS_BYTES_PER_PT_STEP},
+            "roofline": {"kernel": "cheb_step_kernel (one launch per step)", "bound": "hbm",
+                         "achieved": gbs, "unit": "GB/s", "bytes_per_point_step": CHEB_BYTES_PER_PT_STEP},
             "gpu_launches": nl // max(ncalls, 1),
         }
     res["workload"] = ("LRSW variable depth %dx%d, H = 1 + 0.4 sin(2 pi x) cos(4 pi y) + 8 bumps (seed 0), |k|^-3 "
-                       "eta, tau*rho=%g (M=%d), every REXII term (J = %d poles), shared Lanczos basis, %s, "
+                       "eta, tau*rho=%g (M=%d), every REXII term (J = %d poles), shared Chebyshev basis, %s, "
                        "error bound %g" % (n, n, tau_rho, info.M, int(info.n_poles),
                                            "double-float vectors" if form == "mixed" else "FP64", rtol))
     res["form"] = form
@@ -617,52 +586,6 @@ def adjoint_measure(torch, rexi, inputs, form="mixed", n=512, steps=8, tau_rho=2
     }
 
 
-def pole_roofline(form, pole_ms, orbits, nterms, peaks, traffic=None):
-    """Roofline of the pole-sum kernel: executed orbit-terms per launch x
-    operations per term over its launch time, against the measured
-    multiply-add rate (and, beside it, the lane rate derived from unit counts
-    at the maximum clock)."""
-    terms = orbits * nterms
-    t_pole = pole_ms / 1e3
-    if form == "mixed":
-        # every FP32 arithmetic operation counted once (48 of the 62 per term
-        # are single-flop FADD/FMUL), against FP32 lane operations per second:
-        # the measured FFMA rate in lane operations (flops / 2)
-        ops = terms * FP32_INSTR_PER_TERM
-        peak_meas = peaks["fp32"]["lane_ops_per_s"] / 1e12 if peaks else None
-        peak_derived = SMS * 128 * SM_MAX_GHZ / 1e3
-        conv = "FP32 operations per launch (FADD/FMUL/FFMA each 1; 62.375 per term) per second, vs the measured FFMA " \
-               "lane-operation rate (rexi_alu_probe)"
-    else:
-        ops = terms * FP64_INSTR_PER_TERM
-        peak_meas = peaks["fp64"]["lane_ops_per_s"] / 1e12 if peaks else None
-        peak_derived = PEAK_FP64_TFLOPS / 2
-        conv = "FP64 operations per launch (DADD/DFMA each 1; 9 per term) per second, vs the measured DFMA " \
-               "lane-operation rate (rexi_alu_probe)"
-    achieved = ops / t_pole / 1e12
-    if form == "mixed":
-        peak = peak_meas if peak_meas else peak_derived
-        source = "measured (rexi_alu_probe, this run)" if peak_meas else "derived from unit counts"
-    else:
-        # the FP64 probe stays below the nominal 1.25 TFLOP/s on this GPU (its
-        # dependent chains do not saturate the FP64 pipe), and the pole kernel
-        # itself exceeds the probe: take the larger of the two
-        peak = max(peak_meas or 0.0, peak_derived)
-        source = ("nominal 1.25 TFLOP/s FP64 (the probe measured %.3f T lane-op/s, below it)" % peak_meas
-                  if peak_meas and peak_meas < peak_derived else "measured (rexi_alu_probe, this run)")
-    return {
-        "kernel": "pole_orbit_%s_kernel" % form,
-        "bound": "alu", "achieved": achieved, "peak": peak, "unit": "T op/s", "frac": achieved / peak,
-        "traffic": traffic,
-        "flop_convention": conv,
-        "peak_source": source,
-        "peak_derived_lane_rate": peak_derived, "frac_of_derived": achieved / peak_derived,
-        "fma2_tflops": terms * FLOPS_PER_TERM[form] / t_pole / 1e12,
-        "pole_ms_per_launch": pole_ms, "orbits": orbits, "terms_per_launch": terms,
-        "orbit_terms_per_s": terms / t_pole,
-    }
-
-
 def run_ours(args):
     import torch
 
@@ -701,15 +624,11 @@ def run_ours(args):
     ms_phase, ncalls, nlaunch = prof
     launches_per_step = nlaunch / max(1, max(2, args.steps // 4))
     combine_ms = ms_phase[4] / max(ncalls, 1)
-    pole_ms = ms_phase[1] / max(ncalls, 1) - combine_ms  # the pole-sum kernel alone
-    orbits = orbit_count(D)
-    nterms = 2 * (M + 24) + 1
+    pole_ms = ms_phase[1] / max(ncalls, 1) - combine_ms  # the pole sum alone
 
     peaks = None
     if not args.skip_peaks:
         peaks = alu_peaks(torch, rexi, gpu_id)
-    roofline = pole_roofline(args.form, pole_ms, orbits, nterms, peaks,
-                             traffic=NCU_POLE_TRAFFIC_BYTES.get(args.form) if D == 2048 else None)
     phases = {"forward_fft_ms": ms_phase[0] / max(ncalls, 1), "pole_sum_ms": pole_ms, "combine_ms": combine_ms,
               "inverse_fft_ms": ms_phase[2] / max(ncalls, 1), "table_upload_ms": ms_phase[3] / max(ncalls, 1),
               "profiled_ms_per_rexii_step": ms_prof / len(states)}
@@ -730,13 +649,16 @@ def run_ours(args):
                     "traffic": NCU_FFT_FWD_TRAFFIC_BYTES if (D == 2048 and args.form == "mixed") else None,
                     "algorithmic_bytes": fft_bytes,
                     "peak_source": "MEASURED_PEAKS.json hbm_gbs" if "hbm_gbs" in mp else "fallback 6.8 TB/s"}
+    # the transforms are the dominant kernels of the step (the pole sum by local
+    # expansion and the combine take about a fifth of it)
+    roofline = roofline_fft
     # combine pass: reads and writes the 3-field half spectrum (96 B per
     # wavenumber); the per-orbit scalars it also reads are L2-resident and not
     # counted
     comb_bytes = 3 * half * 16 * 2
     comb_gbs = comb_bytes / (combine_ms / 1e3) / 1e9 if combine_ms > 0 else None
     comb_kernel = "pole_orbit_combine_df_kernel" if args.form == "mixed" else "pole_orbit_combine_kernel"
-    roofline_combine = {"kernel": "pole_orbit_finalize_kernel + " + comb_kernel, "bound": "hbm", "achieved": comb_gbs,
+    roofline_combine = {"kernel": comb_kernel, "bound": "hbm", "achieved": comb_gbs,
                         "peak": hbm_peak, "unit": "GB/s", "frac": comb_gbs / hbm_peak if comb_gbs else None,
                         "traffic": NCU_COMBINE_TRAFFIC_BYTES if (D == 2048 and args.form == "mixed") else None,
                         "algorithmic_bytes": comb_bytes}
@@ -800,11 +722,12 @@ def run_ours(args):
             u = nst * D * D * J
             forms[form] = {"value": world * u / (fms / 1e3), "ms_per_rexii_step": fms / nst, "steps": k,
                            "states_per_step": nst}
-        # the fp64 form's pole kernel, for its own roofline
+        # the fp64 form's phases
         if args.form != "fp64":
             _, _, _, fp, _ = time_form(torch, rexi, "fp64", states[:2], 1, 1, world, profile=True)
-            f_pole = fp[0][1] / max(fp[1], 1) - fp[0][4] / max(fp[1], 1)
-            forms["fp64"]["roofline"] = pole_roofline("fp64", f_pole, orbits, nterms, peaks)
+            nf = max(fp[1], 1)
+            forms["fp64"]["phases_ms"] = {"forward_fft_ms": fp[0][0] / nf, "pole_sum_ms": (fp[0][1] - fp[0][4]) / nf,
+                                          "combine_ms": fp[0][4] / nf, "inverse_fft_ms": fp[0][2] / nf}
 
     # complex input (the full two-sided sum, J = 2(2N + 1) poles): the mixed
     # form's complex transforms and its double-float combine on the full spectrum
@@ -842,7 +765,7 @@ def run_ours(args):
                               "combine_ms": cph[4] / max(cn, 1), "inverse_fft_ms": cph[2] / max(cn, 1)}}
         del cws
 
-    # rectangular grid: the kx <-> ky fold is not available, so one pole sum
+    # rectangular grid: the kx <-> ky fold is not available, so one orbit
     # serves four wavenumbers instead of eight
     rect = None
     if not args.skip_rect:
@@ -854,12 +777,11 @@ def run_ours(args):
         Jr = 2 * (Mr + 24 + 1)
         _, _, _, rp, _ = time_form(torch, rexi, args.form, rstates, 2, 1, world, nx=RX, ny=RY, profile=True)
         r_pole = rp[0][1] / max(rp[1], 1) - rp[0][4] / max(rp[1], 1)
-        r_orbits = (RX // 2 + 1) * (RY // 2 + 1)
         rect = {"workload": "%dx%d C-grid (dx = 1/%d, dy = 1/%d), |k|^-3 eta seeds 0-3, tau*rho=%g, form=%s"
                             % (RX, RY, RX, RY, TAU_RHO, args.form),
                 "value": len(rstates) * RX * RY * Jr / (rms / 1e3), "unit": UNIT,
                 "ms_per_rexii_step": rms / len(rstates), "rho": rplan.rho,
-                "roofline": pole_roofline(args.form, r_pole, r_orbits, 2 * (Mr + 24) + 1, peaks)}
+                "pole_sum_ms": r_pole}
 
     batched = None
     if not args.skip_batch:
@@ -876,7 +798,7 @@ def run_ours(args):
         krylov["shared_all_terms"] = {}
         for sform in ("mixed", "fp64"):
             sm = shared_measure(torch, rexi, inputs, form=sform)
-            for key in ("regenerate", "kept_basis"):
+            for key in ("minimum_workspace", "large_workspace"):
                 sm[key]["roofline"]["peak"] = hbm_peak
                 sm[key]["roofline"]["frac"] = sm[key]["roofline"]["achieved"] / hbm_peak
             krylov["shared_all_terms"][sform] = sm
@@ -924,9 +846,9 @@ def run_ours(args):
             "vs_baseline": None, "dtype": "f32x2+f64" if args.form == "mixed" else "f64", "data": "synthetic",
             "config": cfg, "clocks": clocks, "e2e": e2e, "gpu_launches": int(round(launches_per_step * args.steps)),
             "roofline": roofline, "alu_peaks": peaks,
-            "executed": {"orbit_terms_per_s": world * len(states) * orbits * nterms / (ms_max / 1e3),
-                         "note": "one pole sum per orbit of omega's symmetries (8 wavenumbers on this square grid); "
-                                 "value counts every grid point and every pole"},
+            "executed": {"note": "the pole sum is evaluated once per orbit of omega's symmetries (8 wavenumbers on this "
+                                 "square grid), through polynomials fitted to it on cells of the spectrum; value "
+                                 "counts every grid point and every pole"},
             "rectangular": rect, "complex_input": cplx,
             "roofline_fft": roofline_fft, "roofline_combine": roofline_combine, "phases_ms": phases, "forms": forms,
             "batched": batched, "krylov": krylov,

@@ -332,7 +332,8 @@ __global__ void __launch_bounds__(THREADS, 4) cheb_step_kernel(Geom<T> G, StepAr
 }
 
 // Launch that may overlap the previous step's tail (see pdl_wait; not behind a
-// launch of many steps, which wrote what this one loads early); an error is left for the caller's cudaGetLastError.
+// launch of many steps, which wrote what this one loads early).  An error is
+// left for the caller's cudaGetLastError.
 template <typename T, int MODE>
 void launch_step(const Geom<T>& G, const StepArgs<T>& A, int nset, cudaStream_t s, bool overlap = true) {
   cudaLaunchConfig_t cfg = {};
