@@ -457,7 +457,8 @@ def shared_measure(torch, rexi, inputs, rtol=1e-10, reps=3, n=None, tau_rho=None
             "phases_ms": {"steps": pass1, "last_step": ph[2] / max(ncalls, 1), "setup": ph[3] / max(ncalls, 1)},
             "energy_drift": abs(en(o) / en(xn) - 1.0),
             "roofline": {"kernel": "cheb_step_kernel (one launch per step)", "bound": "hbm",
-                         "achieved": gbs, "unit": "GB/s", "bytes_per_point_step": CHEB_BYTES_PER_PT_STEP},
+                         "achieved": gbs, "unit": "GB/s", "bytes_per_point_step": CHEB_BYTES_PER_PT_STEP,
+                         "note": "bytes that a step touches; part of them stay in L2 from step to step"},
             "gpu_launches": nl // max(ncalls, 1),
         }
     res["workload"] = ("LRSW variable depth %dx%d, H = 1 + 0.4 sin(2 pi x) cos(4 pi y) + 8 bumps (seed 0), |k|^-3 "
