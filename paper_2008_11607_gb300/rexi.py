@@ -245,10 +245,21 @@ def alu_probe(kind, blocks, iters, out, stream=None):
     return blocks * 256 * 256 * iters * 2 * (2 if k == 2 else 1)
 
 
-def _own(t, stream):
-    """A tensor allocated here for a call on `stream`: its memory is not reused before that stream is done."""
-    if stream is not None:
-        t.record_stream(stream)
+def _made_on(stream, make, returned=False):
+    """make(): a tensor that a call allocates for itself, allocated (and filled) on
+    the stream that the call runs on, so that neither what the current stream still
+    has queued nor the tensor's release can touch it out of order.  ``returned``:
+    the caller, on the current stream, keeps it."""
+    import torch
+
+    if stream is None:
+        return make()
+    if not isinstance(stream, torch.cuda.Stream):
+        stream = torch.cuda.ExternalStream(stream.cuda_stream)
+    with torch.cuda.stream(stream):
+        t = make()
+    if returned:
+        t.record_stream(torch.cuda.current_stream(t.device))
     return t
 
 
@@ -353,9 +364,9 @@ class Plan:
         import torch
 
         if out is None:
-            out = _own(torch.empty_like(state), stream)
+            out = _made_on(stream, lambda: torch.empty_like(state), returned=True)
         if workspace is None:
-            workspace = _own(self.workspace(dt, tol, real_input, device=state.device), stream)
+            workspace = _made_on(stream, lambda: self.workspace(dt, tol, real_input, device=state.device))
         info = rexi_step_info() if want_info else None
         st = self._lib.rexi_step(self._h, _ptr(state), _ptr(out), dt, tol, int(real_input), int(terms[0]),
                                  int(terms[1]), _ptr(workspace), workspace.numel(), _stream_handle(stream),
@@ -377,7 +388,7 @@ class Plan:
         With blocking=False the copies and the step are only enqueued on ``stream``
         (rexi_step_host_async): ``out_host`` is ready once the stream gets there."""
         if workspace is None:
-            workspace = self.workspace_host(dt, tol, real_input)
+            workspace = _made_on(stream, lambda: self.workspace_host(dt, tol, real_input))
         if blocking:
             st = self._lib.rexi_step_host(self._h, ctypes.c_void_p(state_host.data_ptr()),
                                           ctypes.c_void_p(out_host.data_ptr()), dt, tol, int(real_input),
@@ -409,9 +420,11 @@ class Plan:
         import torch
 
         if grad is None:
-            grad = torch.zeros((self.ny, self.nx), dtype=torch.float64, device=state.device)
+            grad = _made_on(stream, lambda: torch.zeros((self.ny, self.nx), dtype=torch.float64,
+                                                        device=state.device), returned=True)
         if workspace is None:
-            workspace = _own(self.workspace(dt, tol, real_input, device=state.device, grad_depth=True), stream)
+            workspace = _made_on(stream, lambda: self.workspace(dt, tol, real_input, device=state.device,
+                                                                grad_depth=True))
         info = rexi_step_info() if want_info else None
         st = self._lib.rexi_step_grad_depth(self._h, _ptr(state), _ptr(grad_out), _ptr(grad), dt, tol,
                                             int(real_input), _ptr(workspace), workspace.numel(),
@@ -424,11 +437,12 @@ class Plan:
         import torch
 
         if grad is None:
-            grad = torch.zeros((self.ny, self.nx), dtype=torch.float64, device=state.device)
+            grad = _made_on(stream, lambda: torch.zeros((self.ny, self.nx), dtype=torch.float64,
+                                                        device=state.device), returned=True)
         if workspace is None:
             n = max(self.workspace_size(dt, tol, real_input), self.workspace_size(dt, tol, real_input, grad_depth=True))
-            workspace = _own(torch.empty(n, dtype=torch.uint8, device=state.device), stream)
-        out = _own(torch.empty_like(grad_out), stream)
+            workspace = _made_on(stream, lambda: torch.empty(n, dtype=torch.uint8, device=state.device))
+        out = _made_on(stream, lambda: torch.empty_like(grad_out), returned=True)
         st = self._lib.rexi_step_backward(self._h, _ptr(state), _ptr(grad_out), _ptr(out), _ptr(grad), dt, tol,
                                           int(real_input), _ptr(workspace), workspace.numel(), _stream_handle(stream))
         _check(st, "rexi_step_backward")
@@ -438,9 +452,9 @@ class Plan:
         import torch
 
         if out is None:
-            out = _own(torch.empty_like(grad_out), stream)
+            out = _made_on(stream, lambda: torch.empty_like(grad_out), returned=True)
         if workspace is None:
-            workspace = _own(self.workspace(dt, tol, real_input, device=grad_out.device), stream)
+            workspace = _made_on(stream, lambda: self.workspace(dt, tol, real_input, device=grad_out.device))
         st = self._lib.rexi_step_adjoint(self._h, _ptr(grad_out), _ptr(out), dt, tol, int(real_input),
                                          _ptr(workspace), workspace.numel(), _stream_handle(stream))
         _check(st, "rexi_step_adjoint")
@@ -510,9 +524,9 @@ class Batch:
     def step(self, packed_in, packed_out=None, workspace=None, real_input=True, mode=REXI_BATCH_PERSISTENT,
              stream=None):
         if packed_out is None:
-            packed_out = packed_in.new_empty(packed_in.shape)
+            packed_out = _made_on(stream, lambda: packed_in.new_empty(packed_in.shape), returned=True)
         if workspace is None:
-            workspace = self.workspace(packed_in.device)
+            workspace = _made_on(stream, lambda: self.workspace(packed_in.device))
         _check(self._lib.rexi_batch_step(self._h, _ptr(packed_in), _ptr(packed_out), int(real_input),
                                          _ptr(workspace), workspace.numel(), int(mode), _stream_handle(stream)),
                "rexi_batch_step")
