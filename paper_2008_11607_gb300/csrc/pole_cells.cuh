@@ -268,6 +268,25 @@ __device__ __forceinline__ int cell_of(const CellGeom& g, double x, double& t) {
   return k;
 }
 
+// Value at t of a cell's polynomial in double-float, real and imaginary part.  Every
+// coefficient is a pair, as the terms of a direct sum are: monomial coefficient i
+// falls off only like (c/a)^i, 5.13^-i at worst (an FP32 upper half, i >= 8, leaves
+// 1.5e-13 of a single pole's value there, pairs 8e-15; at h = 2 it is 5.6e-11 of the
+// whole sum against 7e-14).
+__device__ __forceinline__ void cell_horner(const float4* __restrict__ p, double t, float2& ar, float2& ai) {
+  const float2 td = df_from_double(t);
+  const float4 top = p[kCellP - 1];
+  ar = make_float2(top.x, top.y);
+  ai = make_float2(top.z, top.w);
+#pragma unroll
+  for (int i = kCellP - 2; i >= 0; --i) {
+    const float4 v = p[i];
+    const float2 pr = f_mul(ar.x, ar.y, td.x, td.y), pi = f_mul(ai.x, ai.y, td.x, td.y);
+    ar = f_add(v.x, v.y, pr.x, pr.y);
+    ai = f_add(v.z, v.w, pi.x, pi.y);
+  }
+}
+
 // fin[o] of orbit o from its cell's polynomial.
 template <int KIND, bool CGRID>
 __device__ __forceinline__ void cell_orbit(const CellGeom& g, const void* __restrict__ poly, const SymbolParams& sp,
@@ -276,25 +295,8 @@ __device__ __forceinline__ void cell_orbit(const CellGeom& g, const void* __rest
   double t;
   const int k = cell_of(g, tau * om.x, t);
   if (KIND == kOrbitDf) {
-    // Horner's rule: the upper half of the coefficients (at most 10.36^-8 =
-    // 7e-9 of the result) in FP32, the lower half in double-float
-    const float4* p = static_cast<const float4*>(poly) + (size_t)k * kCellP;
-    const float2 td = df_from_double(t);
-    float hr = p[kCellP - 1].x, hi = p[kCellP - 1].z;
-#pragma unroll
-    for (int i = kCellP - 2; i >= kCellP / 2; --i) {
-      const float4 v = p[i];
-      hr = fmaf(hr, td.x, v.x);
-      hi = fmaf(hi, td.x, v.z);
-    }
-    float2 ar = make_float2(hr, 0.f), ai = make_float2(hi, 0.f);
-#pragma unroll
-    for (int i = kCellP / 2 - 1; i >= 0; --i) {
-      const float4 v = p[i];
-      const float2 pr = f_mul(ar.x, ar.y, td.x, td.y), pi = f_mul(ai.x, ai.y, td.x, td.y);
-      ar = f_add(v.x, v.y, pr.x, pr.y);
-      ai = f_add(v.z, v.w, pi.x, pi.y);
-    }
+    float2 ar, ai;
+    cell_horner(static_cast<const float4*>(poly) + (size_t)k * kCellP, t, ar, ai);
     const float2 iw = df_from_double(om.y);
     const float2 d = f_subf(df_from_double(R0.x), ar);
     OrbitScalarsDF out;

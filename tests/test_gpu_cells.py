@@ -62,3 +62,26 @@ def test_cells_against_direct_slices(case, form):
     still = plan.step(x, 0.0, real_input=real, workspace=ws).cpu().numpy()
     if coefs != "rexi":
         assert rel_l2(still, np.asarray(x.cpu())) < 1e-10
+
+
+@pytest.mark.parametrize("h", [1.0, 2.0])
+def test_wide_spacing_against_fp64(h):
+    """Cells of half-width 1 and 2: the mixed form against the FP64 form, within the rounding of both
+    term sums and of the transforms (the error model of tests/gpu_util.py)."""
+    torch = torch_cuda()
+    from paper_2008_11607_gb300 import rexi
+    from tests.gpu_util import fft_rounding_bound, pole_rounding_bound
+
+    nx, ny, tau_rho = 256, 250, 200.0
+    x = to_dev(torch, inputs.white_real_state(nx, ny, 3))
+    out, launches, tol = {}, {}, 0.0
+    for form in ("fp64", "mixed"):
+        plan = rexi.Plan(nx, ny, form=form, h=h)
+        dt = tau_rho / plan.rho
+        plan.set_profiling(True)
+        out[form], info = plan.step(x, dt, want_info=True)
+        launches[form] = plan.read_profile()[2]
+        plan.step(x, dt, terms=(0, 8))
+        assert plan.read_profile()[2] < launches[form]  # the whole sum took the cells
+        tol += pole_rounding_bound(form, tau_rho, h, info.M) + fft_rounding_bound(form, nx, ny)
+    assert rel_l2(out["mixed"].cpu().numpy(), out["fp64"].cpu().numpy()) < tol
