@@ -282,6 +282,15 @@ rexi_status rexi_plan_set_krylov(rexi_plan_t plan, double rtol, int32_t max_iter
 enum { REXI_KRYLOV_CG = 0, REXI_KRYLOV_SHARED = 1 };
 rexi_status rexi_plan_set_krylov_method(rexi_plan_t plan, int32_t method);
 
+/* Shared-Krylov steps on grids that fit the multiprocessors' shared memory run
+ * in one launch whose blocks poll each other's edge values.  A wait of more than
+ * `polls` polls (default 2^20, about a second, where waits last microseconds;
+ * at most that; 0: every wait gives up) ends the launch: the call's outputs are
+ * NaN, its depth gradient is not added, and, as the call has returned by then,
+ * the plan's next call (rexi_step_host: the call itself) returns REXI_ETIMEOUT
+ * instead of its own work, once.  REXI_EUNSUPPORTED on constant-depth plans. */
+rexi_status rexi_plan_set_edge_polls(rexi_plan_t plan, int32_t polls);
+
 /* Bytes of device workspace rexi_step and rexi_step_adjoint need for this
  * plan, dt and tol. */
 rexi_status rexi_workspace_size(rexi_plan_t plan, double dt, double tol, int32_t real_input,

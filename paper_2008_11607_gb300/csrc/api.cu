@@ -409,6 +409,14 @@ rexi_status rexi_plan_set_krylov_method(rexi_plan_t p, int32_t method) {
   return REXI_OK;
 }
 
+rexi_status rexi_plan_set_edge_polls(rexi_plan_t p, int32_t polls) {
+  g_err[0] = 0;
+  if (!p || polls < 0 || polls > 1 << 20) return fail(REXI_EINVAL, "polls must be in [0, 2^20]");
+  if (!p->depth) return fail(REXI_EUNSUPPORTED, "edge polls need a variable-depth plan");
+  p->kry.edge_polls = polls;
+  return REXI_OK;
+}
+
 rexi_status rexi_plan_set_krylov(rexi_plan_t p, double rtol, int32_t max_iters, int32_t term_batch) {
   g_err[0] = 0;
   if (!p || !(rtol > 0.0 && rtol < 1.0) || max_iters < 1 || term_batch < 1)
@@ -974,7 +982,7 @@ rexi_status rexi_step_host(rexi_plan_t p, const void* in_host, void* out_host, d
   rexi_status st = step_host_enqueue(p, in_host, out_host, dt, tol, real_input, ws, ws_bytes, stream, info);
   if (st != REXI_OK) return st;
   CUDA_TRY(cudaStreamSynchronize(static_cast<cudaStream_t>(stream)), "stream synchronise");
-  return REXI_OK;
+  return p->depth ? krylov_pending(&p->kry) : REXI_OK;
 }
 
 rexi_status rexi_step_host_async(rexi_plan_t p, const void* in_host, void* out_host, double dt, double tol,

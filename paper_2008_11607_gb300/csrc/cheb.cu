@@ -218,7 +218,7 @@ struct StepArgs {
   double* grad;      // last: the depth gradient
   const double* w;
   int adjoint, real_out;
-  const unsigned* bad;  // last: nonzero where an earlier launch gave up (the result is then NaN)
+  const unsigned* bad;  // last: nonzero where an earlier launch gave up: out is NaN, grad untouched
 };
 
 // One step of the recurrence on a tile of TX x TY points, two rows per thread.
@@ -263,7 +263,8 @@ __global__ void __launch_bounds__(THREADS, 4) cheb_step_kernel(Geom<T> G, StepAr
   }
   T dk = T{};
   if (!FWD) dk = *A.d;
-  if (LAST && A.bad && *A.bad) dk = u_from<T>(nan(""));
+  const bool gone = LAST && A.bad && *A.bad;
+  if (gone) dk = u_from<T>(nan(""));
   cp_async_wait_all();
   __syncthreads();
   const T cu = HALF ? u_half(G.cu) : G.cu, gu = HALF ? u_half(G.gu) : G.gu;
@@ -300,12 +301,11 @@ __global__ void __launch_bounds__(THREADS, 4) cheb_step_kernel(Geom<T> G, StepAr
       }
       if (FWD) A.s[id] = u_norm(s);
       if (GRAD) {
-        T es = LAST ? u_half(e) : e;
-        if (LAST && A.bad && *A.bad) es = dk;
+        const T es = LAST ? u_half(e) : e;
         const T t = u_norm(u_madd(A.first ? T{} : A.acc[id], es, ps[r]));
         if (MODE == kGrad)
           A.acc[id] = t;
-        else
+        else if (!gone)
           A.grad[id] -= A.w[id] * u_to_double(t);
       }
       if (MODE == kSumLast || (MODE == kGradLast && A.out)) {
@@ -371,6 +371,8 @@ void launch_step(const Geom<T>& G, const StepArgs<T>& A, int nset, cudaStream_t 
 struct Exchange {
   ulonglong2 *col, *row;  // [parity][set][3][strip][ny], [parity][set][3][group][nx]
   unsigned* bad;          // a wait ran out
+  unsigned* host_bad;     // the same for the host (KrylovSettings::gave_up)
+  int polls;              // of one wait before a warp gives up
 };
 enum { kColE = 0, kColV = 1, kColU = 2, kRowE = 0, kRowU = 1, kRowV = 2 };
 
@@ -403,9 +405,12 @@ __device__ __forceinline__ ulonglong2 ld_edge(const ulonglong2* p) {
 __device__ __forceinline__ bool arrived(ulonglong2 w, unsigned flag) {
   return (unsigned)(w.x >> 32) == flag && (unsigned)(w.y >> 32) == flag;
 }
-// Polls of one wait before a warp gives up (about a second; a warp's neighbours are
-// resident with it, so a wait lasts microseconds).
-constexpr int kPollLimit = 1 << 20;
+// Out of line: its stores inside the poll loop cost 0.8% of a 512^2 step.
+__device__ __noinline__ void give_up(const Exchange& X, unsigned* dead) {
+  *(volatile unsigned*)X.bad = 1u;
+  *(volatile unsigned*)X.host_bad = 1u;
+  *(volatile unsigned*)dead = 1u;
+}
 
 template <typename T>
 struct ManyArgs {
@@ -550,9 +555,8 @@ __global__ void __launch_bounds__(32 * (kMaxComputeWarps + kCommWarps), 1) cheb_
             b[dst[m]] = unpack<T>(w[m]);
             left &= ~(1u << m);
           }
-        if (n >= kPollLimit || ((n & 1023) == 1023 && *(volatile unsigned*)A.X.bad)) {
-          *(volatile unsigned*)A.X.bad = 1u;
-          *(volatile unsigned*)&dead = 1u;
+        if (n >= A.X.polls || ((n & 1023) == 1023 && *(volatile unsigned*)A.X.bad)) {
+          give_up(A.X, &dead);
           return;
         }
       }
@@ -719,8 +723,12 @@ ManyPlan many_plan(int nx, int ny, int nset, int sms, bool grad, size_t exchange
   }
   return p;
 }
-cudaError_t exchange_at(const ManyPlan& p, int nx, int ny, int nset, void* base, Exchange* X, cudaStream_t s) {
+cudaError_t exchange_at(const ManyPlan& p, const KrylovSettings* k, int nset, void* base, Exchange* X,
+                        cudaStream_t s) {
+  const int nx = k->nx, ny = k->ny;
   char* b = static_cast<char*>(base);
+  X->host_bad = k->gave_up;
+  X->polls = k->edge_polls;
   X->bad = reinterpret_cast<unsigned*>(b);
   X->col = reinterpret_cast<ulonglong2*>(b + 256);
   X->row = X->col + (size_t)2 * nset * 3 * p.ns * ny;
@@ -925,7 +933,7 @@ rexi_status step_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
   bool many = mp.blocks && p.K > 2;
   if (many) {
     ManyArgs<T> Q = {};
-    e = exchange_at(mp, k->nx, k->ny, nset, b.exchange, &Q.X, s);
+    e = exchange_at(mp, k, nset, b.exchange, &Q.X, s);
     Q.b1 = bA;
     Q.o1 = bA;
     Q.o2 = bB;
@@ -992,7 +1000,7 @@ rexi_status grad_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
   ManyArgs<T> Q = {};
   Q.H = depth_table(k, T{});
   Q.steps = p.K - 1;
-  if (many && e == cudaSuccess) e = exchange_at(mp, k->nx, k->ny, 1, b.exchange, &Q.X, s);
+  if (many && e == cudaSuccess) e = exchange_at(mp, k, 1, b.exchange, &Q.X, s);
   // forward: P_0 in bA, P_1 in bB, then each P_{k+1} over P_{k-1}; s_k for k < K
   Geom<T> G = make_geom<T>(k, dt, p);
   if (e == cudaSuccess) e = init(G, k, f_in, 0, bA, static_cast<T*>(nullptr), d, S, 1, s, &launches);
@@ -1034,6 +1042,7 @@ rexi_status grad_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
   A.H = depth_table(k, T{});
   A.acc = static_cast<T*>(b.acc);
   A.first = 1;
+  A.bad = Q.X.bad;  // of either launch of many steps (null: no exchange was set up)
   const T *b1, *b2;
   if (many) {
     Q.b1 = bA;
@@ -1049,11 +1058,9 @@ rexi_status grad_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
     if (e != cudaSuccess) return failed(e);
     b1 = bA;
     b2 = bB;
-    A.bad = Q.X.bad;
     launches += many;
   }
   if (!many) {
-    A.bad = nullptr;
     clenshaw<T, kGrad>(G, A, p.K, d, bA, bB, sf, 1, s, &b1, &b2);
     launches += p.K - 1;
   }

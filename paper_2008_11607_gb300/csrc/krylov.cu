@@ -986,12 +986,14 @@ rexi_status krylov_init(KrylovSettings* k, int nx, int ny, double Lx, double Ly,
   k->Hdf = reinterpret_cast<float2*>(mem + al256(nk * sizeof(double)) + 2 * al256(nk * sizeof(float)));
   k->wdf = reinterpret_cast<float2*>(mem + al256(nk * sizeof(double)) + 2 * al256(nk * sizeof(float)) +
                                      al256(nk * sizeof(float2)));
-  if (cudaMallocHost(reinterpret_cast<void**>(&k->pinned), 8 * sizeof(double)) != cudaSuccess ||
+  if (cudaMallocHost(reinterpret_cast<void**>(&k->pinned), 9 * sizeof(double)) != cudaSuccess ||
       cudaEventCreateWithFlags(&k->ev[0], cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&k->ev[1], cudaEventDisableTiming) != cudaSuccess) {
     set_last_error("pinned buffer or event creation failed");
     return REXI_ECUDA;
   }
+  k->gave_up = reinterpret_cast<unsigned*>(k->pinned + 8);
+  *k->gave_up = 0u;
   depth_tables<<<(unsigned)((nk + 255) / 256), 256>>>(depth, nk, g, k->w64, k->H32, k->w32);
   if (lanczos_tables(k) != REXI_OK) return REXI_ECUDA;
   if (cudaDeviceSynchronize() != cudaSuccess) {
@@ -1010,6 +1012,13 @@ void krylov_destroy(KrylovSettings* k) {
     if (e) cudaEventDestroy(e);
     e = nullptr;
   }
+}
+
+rexi_status krylov_pending(KrylovSettings* k) {
+  if (!k->gave_up || !__atomic_exchange_n(k->gave_up, 0u, __ATOMIC_ACQ_REL)) return REXI_OK;
+  set_last_error("shared-Krylov method: an earlier call of this plan gave up waiting for edge values between "
+                 "blocks; its outputs are NaN and its depth gradient was not added");
+  return REXI_ETIMEOUT;
 }
 
 size_t krylov_workspace_bytes(const KrylovSettings* k, int M, int real_input, int form) {
@@ -1308,6 +1317,8 @@ bool overlaps(const void* a, const void* b, size_t bytes) {
 rexi_status krylov_step(KrylovSettings* k, int form, double h, int M, const void* in, void* out, double dt,
                         int real_input, int term_begin, int term_end, void* ws, size_t ws_bytes, cudaStream_t s,
                         rexi_step_info* info, bool adjoint, const KrylovHooks& hooks) {
+  rexi_status st = krylov_pending(k);
+  if (st != REXI_OK) return st;
   if (k->method == 1)
     return krylov_step_lanczos(k, form, h, M, in, out, dt, real_input, term_begin, term_end, ws, ws_bytes, s, info,
                                adjoint, hooks);
@@ -1318,7 +1329,7 @@ rexi_status krylov_step(KrylovSettings* k, int form, double h, int M, const void
   }
   KrylovRun run;
   // adjoint: r(tau A)^H = r(tau A^T) = W r(-tau A) W^{-1} with W = diag(g/H, 1, 1)
-  rexi_status st = run.setup(k, form, h, M, adjoint ? -dt : dt, real_input, term_begin, term_end, ws, ws_bytes, s,
+  st = run.setup(k, form, h, M, adjoint ? -dt : dt, real_input, term_begin, term_end, ws, ws_bytes, s,
                              &hooks);
   if (st != REXI_OK) return st;
   const double2* src = static_cast<const double2*>(in);
@@ -1368,12 +1379,14 @@ rexi_status krylov_grad_depth(KrylovSettings* k, int form, double h, int M, cons
                               double* grad_depth, void* grad_in, double dt, int real_input, void* ws, size_t ws_bytes,
                               cudaStream_t s, rexi_step_info* info, const KrylovHooks& hooks, bool* grad_in_done) {
   *grad_in_done = false;
+  rexi_status st = krylov_pending(k);
+  if (st != REXI_OK) return st;
   if (k->method == 1 && real_input)
     return krylov_grad_depth_lanczos(k, form, h, M, f_in, g_out, grad_depth, grad_in, dt, ws, ws_bytes, s, info, hooks,
                                      grad_in_done);
   const size_t nk = (size_t)k->nx * k->ny, n3 = 3 * nk;
   KrylovRun run;
-  rexi_status st = run.setup(k, form, h, M, dt, real_input, 0, -1, ws, ws_bytes, s, &hooks);
+  st = run.setup(k, form, h, M, dt, real_input, 0, -1, ws, ws_bytes, s, &hooks);
   if (st != REXI_OK) return st;
   const unsigned ebl = (unsigned)((n3 + 255) / 256);
   // adjoint right-hand side W^{-1} G

@@ -21,6 +21,10 @@ struct KrylovSettings {
   double rho_op = 0;          // the operator's own bound, whatever rho the plan was given
   int sms = 0;                // multiprocessors of the device
   double* pinned = nullptr;   // small pinned host buffer (convergence checks)
+  // Set (host memory, by the device) when a wait for edge values gave up; reported
+  // by the plan's next call (krylov_pending).
+  unsigned* gave_up = nullptr;
+  int edge_polls = 1 << 20;   // polls of such a wait (about a second; it lasts microseconds)
   cudaEvent_t ev[2] = {nullptr, nullptr};
   void* dev_state = nullptr;  // plan-owned device tables below
   double* w64 = nullptr;      // energy weight g / H (FP64)
@@ -41,6 +45,8 @@ struct KrylovHooks {
 rexi_status krylov_init(KrylovSettings* k, int nx, int ny, double Lx, double Ly, double g, double f,
                         const double* depth, double Hmean);
 void krylov_destroy(KrylovSettings* k);
+// REXI_ETIMEOUT, once, where an earlier call of the plan gave up waiting.
+rexi_status krylov_pending(KrylovSettings* k);
 size_t krylov_workspace_bytes(const KrylovSettings* k, int M, int real_input, int form);
 size_t krylov_grad_workspace_bytes(const KrylovSettings* k, int M, int real_input, int form, double h);
 rexi_status krylov_step(KrylovSettings* k, int form, double h, int M, const void* in, void* out, double dt,

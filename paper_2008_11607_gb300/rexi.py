@@ -77,6 +77,7 @@ SIGNATURES = {
     "rexi_spectral_radius": (_c_int, [_vp, _dp]),
     "rexi_plan_set_krylov": (_c_int, [_vp, _c_dbl, _c_int, _c_int]),
     "rexi_plan_set_krylov_method": (_c_int, [_vp, _c_int]),
+    "rexi_plan_set_edge_polls": (_c_int, [_vp, _c_int]),
     "rexi_plan_set_symbol": (_c_int, [_vp, _c_int]),
     "rexi_plan_set_rho": (_c_int, [_vp, _c_dbl]),
     "rexi_plan_set_coefficients": (_c_int, [_vp, _c_int]),
@@ -340,6 +341,11 @@ class Plan:
         """Variable-depth solver: "cg" (one CG per REXII term) or "shared" (one Lanczos basis for all poles)."""
         code = KRYLOV_METHODS[method] if isinstance(method, str) else int(method)
         _check(self._lib.rexi_plan_set_krylov_method(self._h, code), "rexi_plan_set_krylov_method")
+
+    def set_edge_polls(self, polls=1 << 20):
+        """Polls that a block of a shared-Krylov step waits for a neighbour's edge before the step gives
+        up: NaN outputs, no depth gradient added, REXI_ETIMEOUT from the plan's next call."""
+        _check(self._lib.rexi_plan_set_edge_polls(self._h, int(polls)), "rexi_plan_set_edge_polls")
 
     def krylov_vector_bytes(self, real_input=True):
         """Bytes of one kept Lanczos vector of the shared-Krylov method (extra workspace beyond
