@@ -42,6 +42,7 @@
 
 #include "cheb.h"
 #include "dfloat.cuh"
+#include "recip.cuh"
 
 namespace rexi {
 namespace {
@@ -88,14 +89,6 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---- coefficients ----------------------------------------------------------
-
-// 1 / x for normal FP64 x: hardware seed, r0 (1 + e + e^2) with e = 1 - x r0.
-__device__ __forceinline__ double rcp64(double x) {
-  double r0;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(x));
-  const double e = fma(-x, r0, 1.0);
-  return fma(r0, fma(e, e, e), r0);
-}
 
 constexpr int NT = 128;
 

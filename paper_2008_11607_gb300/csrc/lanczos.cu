@@ -48,6 +48,7 @@
 #include "internal.h"
 #include "krylov.h"
 #include "partials.cuh"
+#include "recip.cuh"
 
 namespace rexi {
 namespace {
@@ -753,25 +754,14 @@ __global__ void lz_finish(const T* acc, double2* out, const double* w, size_t nk
   out[i] = v;
 }
 
-// 1 / x for normal FP64 x: the hardware's approximate FP64 reciprocal r0 as
-// the seed, then r0 (1 + e + e^2) with e = 1 - x r0 (1 / x = r0 / (1 - e)),
-// which leaves a relative error of order e^3, below FP64 rounding: four
-// dependent operations, where a dependent FP64 operation on this GPU waits
-// about a hundred cycles.
-__device__ __forceinline__ double lrcp(double x) {
-  double r0;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(x));
-  const double e = fma(-x, r0, 1.0);
-  return fma(r0, fma(e, e, e), r0);
-}
 // 1 / z for the pivots of the shifted tridiagonal systems (T_k + s_p): every
 // shift lies h |mu| from the line that holds the spectrum of T_k, and each
 // pivot d_j = a_j + s_p - b_j^2 / d_{j-1} keeps at least that distance (the
 // term -b_j^2 / d_{j-1} moves it away from the line, never towards it), so
-// |z|^2 is a normal number for lrcp.  The hardware seed and three FMAs
+// |z|^2 is a normal number for rcp64.  The hardware seed and three FMAs
 // instead of an FP64 division, the longest step of the per-pole recurrences.
 __device__ __forceinline__ double2 crcp(double2 z) {
-  const double r = lrcp(fma(z.x, z.x, z.y * z.y));
+  const double r = rcp64(fma(z.x, z.x, z.y * z.y));
   return make_double2(z.x * r, -z.y * r);
 }
 __device__ __forceinline__ double2 cmuld(double2 a, double2 b) {
@@ -836,7 +826,7 @@ __global__ void __launch_bounds__(BT) lz_bound_part(int np, int G, const double2
     const int cnt = min(BT, pe - p0);
     for (int q = 0; q < cnt; ++q) {
       const double a = lam + ss[q].x, b = ss[q].y;
-      const double r = lrcp(fma(a, a, b * b));
+      const double r = rcp64(fma(a, a, b * b));
       re = fma(r, fma(sw[q].x, a, sw[q].y * b), re);   // Re w / (a + ib)
       im = fma(r, fma(sw[q].y, a, -sw[q].x * b), im);  // Im w / (a + ib)
     }

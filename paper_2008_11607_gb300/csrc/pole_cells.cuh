@@ -228,9 +228,8 @@ __device__ __forceinline__ void cell_poly(const CellGeom& g, const void* table, 
 }
 
 // omega and 1 / omega (0 and 0 at omega = 0) of orbit o.  On the C grid from
-// omega^2 by the hardware's approximate FP64 reciprocal root and a cubic
-// correction, then one residual step for omega: 17 FP64 instructions where
-// the library root and a division take about 45.
+// omega^2 by sqrt_rsqrt64, whose chain is shorter than a library root's and a
+// division's (both sides measured in pole_cells.cu).
 template <bool CGRID>
 __device__ __forceinline__ double2 orbit_omega(const SymbolParams& sp, const OrbitParams& op, int o) {
   int a, b;
@@ -240,14 +239,7 @@ __device__ __forceinline__ double2 orbit_omega(const SymbolParams& sp, const Orb
     const double ax = hx.y * (2.0 * sp.inv_dx), ay = hy.y * (2.0 * sp.inv_dy);
     const double fc = sp.f * hx.x * hy.x;
     const double w2 = fma(sp.g * sp.H, fma(ax, ax, ay * ay), fc * fc);
-    if (w2 > 1e-280 && w2 < 1e280) {
-      double y0;
-      asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(w2));
-      const double e = fma(-w2 * y0, y0, 1.0);
-      const double y = fma(y0 * e, fma(0.375, e, 0.5), y0);
-      const double s = w2 * y;
-      return make_double2(fma(fma(-s, s, w2), 0.5 * y, s), y);
-    }
+    if (w2 > 1e-280 && w2 < 1e280) return sqrt_rsqrt64(w2);
   }
   const double w = symbol_at(sp, a, b).omega;
   return make_double2(w, w > 0.0 ? 1.0 / w : 0.0);

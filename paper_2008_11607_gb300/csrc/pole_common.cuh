@@ -5,6 +5,7 @@
 
 #include "dfloat.cuh"
 #include "internal.h"
+#include "recip.cuh"
 
 namespace rexi {
 
@@ -413,12 +414,6 @@ __device__ __forceinline__ void orbit_rep(const OrbitParams& op, int o, int& a, 
 // Table (per scalar term, 6 doubles): h n, A_re, A_im, B_re, B_im, 0 with
 // A = c1_n h mu, B = c2_n.
 
-__device__ __forceinline__ double rcp_seed(double d) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-  return r;
-}
-
 constexpr int kChunk = 256;  // terms staged in shared memory at a time
 
 // ---------------------------------------------------------------------------
@@ -449,11 +444,7 @@ __device__ __forceinline__ void fp64_term(const double2* e, double x, double q, 
   const double2 e0 = e[0], e1 = e[1], e2 = e[2];
   const double y = x + e0.x;
   const double d = fma(y, y, q);
-  const double r0 = rcp_seed(d);
-  // 1/d = r0 / (1 - e) with e = 1 - d r0; r0 (1 + e + e^2) leaves a relative
-  // error of order e^3 (a Newton-Raphson step plus its next term)
-  const double er = fma(-d, r0, 1.0);
-  const double r = fma(r0, fma(er, er, er), r0);
+  const double r = rcp64(d);
   accr = fma(fma(e1.y, y, e0.y), r, accr);
   acci = fma(fma(e2.x, y, e1.x), r, acci);
 }

@@ -16,8 +16,8 @@
 // applies r(tau B) at every wavenumber with its own symbol.
 //
 // Forms:
-//  * pole_orbit_fp64 / pole_fused_fp64 -- FP64 registers; 1/d by the
-//    rcp.approx seed plus a Newton-Raphson step with its next term in FP64.
+//  * pole_orbit_fp64 / pole_fused_fp64 -- FP64 registers; 1/d by rcp64
+//    (recip.cuh).
 //  * pole_orbit_mixed -- the same sum in double-float
 //    arithmetic (pairs of FP32 values with Dekker/Knuth error-free
 //    transformations: TwoSum, TwoProduct by FMA), FP64 only for the

@@ -18,8 +18,21 @@ __global__ void horner(int n, const double* re, const double* im, const double* 
   cell_horner(p, t[i], ar, ai);
   out[i] = make_double2(df_to_double(ar), df_to_double(ai));
 }
+// out[3 i ..] = rcp64(x[i]) and sqrt_rsqrt64(x[i])
+__global__ void reciprocals(int n, const double* x, double* out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double2 s = sqrt_rsqrt64(x[i]);
+  out[3 * i] = rcp64(x[i]);
+  out[3 * i + 1] = s.x;
+  out[3 * i + 2] = s.y;
+}
 }  // namespace
 
+extern "C" int device_reciprocals(int n, const double* x, double* out) {
+  reciprocals<<<(n + 127) / 128, 128>>>(n, x, out);
+  return (int)cudaDeviceSynchronize();
+}
 extern "C" int device_horner(int n, const double* re, const double* im, const double* t, void* out) {
   horner<<<(n + 127) / 128, 128>>>(n, re, im, t, static_cast<double2*>(out));
   return (int)cudaDeviceSynchronize();

@@ -60,3 +60,19 @@ def test_cell_polynomial_in_pairs(device, name):
         ref = np.polynomial.polynomial.polyval(t.astype(np.longdouble), c.astype(np.longdouble))
         bound = 46 * 2.0 ** -47 * np.polynomial.polynomial.polyval(np.abs(t), np.abs(c))
         assert np.all(np.abs(v - ref) <= bound + 2.0 ** -126)  # and the least that FP32 holds
+
+
+def test_reciprocal_and_roots_over_their_exponents(device):
+    """rcp64 and sqrt_rsqrt64 against NumPy's correctly rounded 1 / x and sqrt(x) in extended
+    precision: one unit in the last place, 2^-52 relative (half of it the final rounding, the
+    rest the residual's rounding and the seed's third-order remainder, 2^-57)."""
+    rng = np.random.default_rng(5)
+    ends = [1.0, 1.0 + 2.0 ** -52, 2.0 - 2.0 ** -52, 1.5, math.sqrt(2.0)]
+    m = np.concatenate([rng.uniform(1.0, 2.0, 100000), np.repeat(ends, 400)])
+    e = np.concatenate([rng.integers(-929, 930, 100000), np.tile(np.linspace(-929, 929, 400).astype(int), len(ends))])
+    x = np.concatenate([np.ldexp(m, e), rng.uniform(0.1, 1e7, 100000)])  # the last: what the sums meet
+    assert x.min() > 1e-280 and x.max() < 1e280
+    got = device("device_reciprocals", len(x), x, out=(len(x), 3))
+    X = x.astype(np.longdouble)
+    for v, ref in zip(got.T, (1.0 / X, np.sqrt(X), 1.0 / np.sqrt(X))):
+        assert np.max(np.abs(v - ref) / ref) <= 2.0 ** -52
