@@ -1184,7 +1184,8 @@ struct KrylovRun {
     return !mixed && tau != 0.0 && k->rho_op > 0.0 && (top * top / q + 1.0) * 0x1p-46 <= 0.25 * k->rtol;
   }
   // The batch's systems in double-float, checked in FP64; *ok: every term is done
-  // (hs holds the outcome), else the FP64 iterations have to follow from cg_init on.
+  // (hs holds the outcome), else the FP64 iterations have to follow from cg_init on,
+  // after the iteration cap too: FP64 may converge a few iterations sooner.
   cudaError_t solve_df(const double2* rhs, int real_rhs, int nb, bool* ok) {
     GeomDf D;
     D.nx = G.nx;
@@ -1227,7 +1228,6 @@ struct KrylovRun {
     *ok = true;
     for (int b = 0; b < nb; ++b) {
       hs[b].iters = hs32[b].iters;
-      if (hs[b].status == 4 && hs32[b].status == 2) hs[b].status = 2;  // the iteration cap
       if (hs[b].status == 4) *ok = false;
     }
     if (!*ok) term_iters = before;

@@ -55,3 +55,25 @@ def test_values_beyond_single_precision_and_the_iteration_cap():
     with pytest.raises(rexi.RexiError) as err:
         plan.step(to_dev(torch, st), dt)
     assert err.value.status == rexi.REXI_ENOCONV
+
+
+def test_iteration_cap_in_double_float_leaves_the_fp64_iterations():
+    """Terms that reach the cap in double-float have the FP64 iterations, under the same cap,
+    before the call gives up: the launches of a call that runs only those (an rtol that
+    double-float cannot reach) come on top of the double-float ones."""
+    from paper_2008_11607_gb300 import rexi
+
+    torch = torch_cuda()
+    nx, ny = 20, 18
+    plan = krylov_plan(torch, nx, ny, inputs.variable_depth(nx, ny, seed=5), rtol=RTOL)
+    dt = 8.0 / plan.rho
+    x = to_dev(torch, inputs.kminus3_field(nx, ny, seed=6))
+    launches = {}
+    for rtol in (RTOL, 1e-14):
+        plan.set_krylov(rtol=rtol, max_iters=3, term_batch=8)
+        plan.set_profiling(True)
+        with pytest.raises(rexi.RexiError) as err:
+            plan.step(x, dt)
+        assert err.value.status == rexi.REXI_ENOCONV
+        launches[rtol] = plan.read_profile()[2]
+    assert launches[RTOL] >= 2 * launches[1e-14]
