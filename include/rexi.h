@@ -352,8 +352,10 @@ rexi_status rexi_step_grad_depth(rexi_plan_t plan, const void* in_dev, const voi
  * rexi_step_adjoint, and dL/dH added to grad_depth as rexi_step_grad_depth.  With
  * the shared-Krylov method and real input the adjoint step is the end of the
  * recurrence that the depth gradient runs, so it comes without one of its own.
- * grad_in_dev must not overlap the other states.  Workspace: the larger of
- * rexi_workspace_size and rexi_workspace_size_grad_depth. */
+ * Otherwise the adjoint step runs first, and grad_depth is as it was when that
+ * fails; grad_in is undefined after an error.  grad_in_dev must not overlap the
+ * other states.  Workspace: the larger of rexi_workspace_size and
+ * rexi_workspace_size_grad_depth. */
 rexi_status rexi_step_backward(rexi_plan_t plan, const void* in_dev, const void* grad_out_dev, void* grad_in_dev,
                                double* grad_depth_dev, double dt, double tol, int32_t real_input,
                                void* workspace_dev, size_t workspace_bytes, void* stream);

@@ -1026,7 +1026,7 @@ rexi_status rexi_plan_read_profile(rexi_plan_t p, double* ms5, int32_t* n_calls,
 namespace {
 rexi_status grad_depth_impl(rexi_plan_t p, const void* in, const void* gout, void* gin, double* grad_depth, double dt,
                             double tol, int32_t real_input, void* ws, size_t ws_bytes, void* stream,
-                            rexi_step_info* info, int* M_out, bool* gin_done) {
+                            rexi_step_info* info) {
   g_err[0] = 0;
   int M = 0;
   rexi_status st = check_step_args(p, in, const_cast<void*>(gout), dt, tol, ws, &M);
@@ -1038,13 +1038,12 @@ rexi_status grad_depth_impl(rexi_plan_t p, const void* in, const void* gout, voi
   hooks.ctx = p;
   hooks.launches = &p->launches;
   st = krylov_grad_depth(&p->kry, p->form, p->h, M, in, gout, grad_depth, gin, dt, real_input, ws, ws_bytes,
-                         static_cast<cudaStream_t>(stream), info, hooks, gin_done);
+                         static_cast<cudaStream_t>(stream), info, hooks);
   if (info) {
     info->M = M;
     info->tau_rho = dt * p->rho;
     info->rho = p->rho;
   }
-  *M_out = M;
   return st;
 }
 }  // namespace
@@ -1052,9 +1051,7 @@ rexi_status grad_depth_impl(rexi_plan_t p, const void* in, const void* gout, voi
 extern "C" rexi_status rexi_step_grad_depth(rexi_plan_t p, const void* in, const void* gout, double* grad_depth,
                                            double dt, double tol, int32_t real_input, void* ws, size_t ws_bytes,
                                            void* stream, rexi_step_info* info) {
-  int M = 0;
-  bool done = false;
-  return grad_depth_impl(p, in, gout, nullptr, grad_depth, dt, tol, real_input, ws, ws_bytes, stream, info, &M, &done);
+  return grad_depth_impl(p, in, gout, nullptr, grad_depth, dt, tol, real_input, ws, ws_bytes, stream, info);
 }
 
 extern "C" rexi_status rexi_step_backward(rexi_plan_t p, const void* in, const void* gout, void* gin,
@@ -1068,11 +1065,7 @@ extern "C" rexi_status rexi_step_backward(rexi_plan_t p, const void* in, const v
   const char *o = static_cast<const char*>(gin), *a = static_cast<const char*>(in), *b = static_cast<const char*>(gout);
   if ((o < a + bytes && a < o + bytes) || (o < b + bytes && b < o + bytes))
     return fail(REXI_EINVAL, "grad_in must not overlap the input or its gradient");
-  bool done = false;
-  st = grad_depth_impl(p, in, gout, gin, grad_depth, dt, tol, real_input, ws, ws_bytes, stream, nullptr, &M, &done);
-  if (st != REXI_OK || done) return st;
-  return krylov_step(&p->kry, p->form, p->h, M, gout, gin, dt, real_input, 0, -1, ws, ws_bytes,
-                     static_cast<cudaStream_t>(stream), nullptr, true, KrylovHooks());
+  return grad_depth_impl(p, in, gout, gin, grad_depth, dt, tol, real_input, ws, ws_bytes, stream, nullptr);
 }
 
 namespace {

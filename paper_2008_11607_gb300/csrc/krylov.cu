@@ -1377,13 +1377,16 @@ rexi_status krylov_step(KrylovSettings* k, int form, double h, int M, const void
 
 rexi_status krylov_grad_depth(KrylovSettings* k, int form, double h, int M, const void* f_in, const void* g_out,
                               double* grad_depth, void* grad_in, double dt, int real_input, void* ws, size_t ws_bytes,
-                              cudaStream_t s, rexi_step_info* info, const KrylovHooks& hooks, bool* grad_in_done) {
-  *grad_in_done = false;
+                              cudaStream_t s, rexi_step_info* info, const KrylovHooks& hooks) {
   rexi_status st = krylov_pending(k);
   if (st != REXI_OK) return st;
   if (k->method == 1 && real_input)
-    return krylov_grad_depth_lanczos(k, form, h, M, f_in, g_out, grad_depth, grad_in, dt, ws, ws_bytes, s, info, hooks,
-                                     grad_in_done);
+    return krylov_grad_depth_lanczos(k, form, h, M, f_in, g_out, grad_depth, grad_in, dt, ws, ws_bytes, s, info, hooks);
+  if (grad_in) {  // before anything is added to the gradient: an adjoint that fails leaves it alone
+    st = krylov_step(k, form, h, M, g_out, grad_in, dt, real_input, 0, -1, ws, ws_bytes, s, nullptr, true,
+                     hooks.launches_only());
+    if (st != REXI_OK) return st;
+  }
   const size_t nk = (size_t)k->nx * k->ny, n3 = 3 * nk;
   KrylovRun run;
   st = run.setup(k, form, h, M, dt, real_input, 0, -1, ws, ws_bytes, s, &hooks);

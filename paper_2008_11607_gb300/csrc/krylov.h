@@ -40,6 +40,12 @@ struct KrylovHooks {
   void (*mark)(void* ctx, int i, cudaStream_t s) = nullptr;
   void* ctx = nullptr;
   int64_t* launches = nullptr;
+  // for a step inside another call: its launches count, its phases are not marked
+  KrylovHooks launches_only() const {
+    KrylovHooks h;
+    h.launches = launches;
+    return h;
+  }
 };
 
 rexi_status krylov_init(KrylovSettings* k, int nx, int ny, double Lx, double Ly, double g, double f,
@@ -61,15 +67,15 @@ size_t lanczos_grad_workspace_bytes(const KrylovSettings* k, int M, double h);
 rexi_status krylov_grad_depth_lanczos(KrylovSettings* k, int form, double h, int M, const void* f_in,
                                       const void* g_out,
                                       double* grad_depth, void* grad_in, double dt, void* ws, size_t ws_bytes,
-                                      cudaStream_t s, rexi_step_info* info, const KrylovHooks& hooks,
-                                      bool* grad_in_done);
+                                      cudaStream_t s, rexi_step_info* info, const KrylovHooks& hooks);
 rexi_status krylov_step_lanczos(KrylovSettings* k, int form, double h, int M, const void* in, void* out, double dt,
                                 int real_input, int term_begin, int term_end, void* ws, size_t ws_bytes,
                                 cudaStream_t s, rexi_step_info* info, bool adjoint, const KrylovHooks& hooks);
 // grad_depth += dL/dH for out = r(dt A(H)) f_in and G = dL/d out.  grad_in
-// (nullable): r(dt A)^H G as well where that comes with it (*grad_in_done).
+// (nullable) = r(dt A)^H G, from the same recurrence where that has it, else by a
+// step of its own before anything is added.
 rexi_status krylov_grad_depth(KrylovSettings* k, int form, double h, int M, const void* f_in, const void* g_out,
                               double* grad_depth, void* grad_in, double dt, int real_input, void* ws, size_t ws_bytes,
-                              cudaStream_t s, rexi_step_info* info, const KrylovHooks& hooks, bool* grad_in_done);
+                              cudaStream_t s, rexi_step_info* info, const KrylovHooks& hooks);
 
 }  // namespace rexi

@@ -1610,8 +1610,7 @@ size_t lanczos_grad_workspace_bytes(const KrylovSettings* k, int M, double h) { 
 rexi_status krylov_grad_depth_lanczos(KrylovSettings* k, int form, double h, int M, const void* f_in,
                                       const void* g_out,
                                       double* grad_depth, void* grad_in, double dt, void* ws, size_t ws_bytes,
-                                      cudaStream_t s, rexi_step_info* info, const KrylovHooks& hooks,
-                                      bool* grad_in_done) {
+                                      cudaStream_t s, rexi_step_info* info, const KrylovHooks& hooks) {
   using cd = std::complex<double>;
   auto mark = [&](int i) {
     if (hooks.mark) hooks.mark(hooks.ctx, i, s);
@@ -1638,7 +1637,6 @@ rexi_status krylov_grad_depth_lanczos(KrylovSettings* k, int form, double h, int
     const rexi_status st =
         cheb_grad(k, cp, form == REXI_FORM_MIXED ? 1 : 0, h, M, f_in, g_out, grad_depth, grad_in, dt, cb, s, hooks,
                   &tail);
-    if (st == REXI_OK) *grad_in_done = grad_in != nullptr;
     if (st == REXI_OK && info) {
       memset(info, 0, sizeof(*info));
       info->N = N;
@@ -1649,6 +1647,12 @@ rexi_status krylov_grad_depth_lanczos(KrylovSettings* k, int form, double h, int
       info->krylov_term_iters = 2 * (int64_t)cp.K;
     }
     if (st != REXI_EUNSUPPORTED) return st;
+  }
+  if (grad_in) {  // before anything is added to the gradient: an adjoint that fails leaves it alone
+    const rexi_status st =
+        krylov_step_lanczos(k, form, h, M, g_out, grad_in, dt, 1, 0, -1, ws, ws_bytes, s, nullptr, true,
+                            hooks.launches_only());
+    if (st != REXI_OK) return st;
   }
   // reduced (real-input) pole set: run on f uses shifts i z_j with beta_j, the run
   // on W^{-1} G uses shifts i conj(z_j) with conj(beta_j)
