@@ -153,16 +153,25 @@ __global__ void __launch_bounds__(NT) cheb_coeffs(const double2* val, int n, dou
   }
 }
 
-// report = (sum_{K < k < n} |d_k|, high word of the largest |input|)
-__global__ void __launch_bounds__(32) cheb_report(const double* d, int K, int n, const unsigned* maxbits,
-                                                  double* report) {
+// report = (sum_{K < k < n} |d_k|, whether the expansion stands), *declined = 1 where
+// it does not.  It stands with a tail within rtol and input that is zero or of a
+// size that the arithmetic holds with room on both sides (exponents of +-room: 64
+// for double-float, 900 for FP64).  Other input, NaN and infinities included, is
+// left to the Lanczos form, which normalises its vectors and reports what is not
+// finite.
+__global__ void __launch_bounds__(32) cheb_report(const double* d, int K, int n, const unsigned* maxbits, double rtol,
+                                                  int room, double* report, unsigned* declined) {
   double a = 0.0;
   for (int k = K + 1 + threadIdx.x; k < n; k += 32) a += fabs(d[k]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
   if (threadIdx.x == 0) {
+    const unsigned hi = *maxbits;  // high word of the largest |input|
+    const int ex = (int)(hi >> 20) - 1023;
+    const bool ok = a <= rtol && (hi == 0u || (ex >= -room && ex <= room));
     report[0] = a;
-    report[1] = (double)*maxbits;
+    report[1] = ok ? 1.0 : 0.0;
+    if (!ok) *declined = 1u;
   }
 }
 
@@ -414,6 +423,7 @@ struct ManyArgs {
   T* acc;            // kGrad: sum of mu_eta s (written)
   int steps, nset, ns, ng, seg_shift;
   unsigned flag0;    // flags of earlier launches on this exchange buffer end here
+  const unsigned* declined;  // nonzero: the expansion does not stand (cheb_report), nothing to do
   Exchange X;
 };
 
@@ -476,7 +486,9 @@ __global__ void __launch_bounds__(32 * (kMaxComputeWarps + kCommWarps), 1) cheb_
     if (GRAD) sA[f] = T{};
   }
   if (threadIdx.x == 0) dead = 0u;
+  const unsigned declined = *A.declined;
   __syncthreads();
+  if (declined) return;
 
   if (warp >= nc) {
     // ---- edges
@@ -778,7 +790,7 @@ struct Scratch {
   double* d;
   float2* d_df;
   double* report;
-  unsigned* maxbits;
+  unsigned *maxbits, *declined;
 };
 size_t al(size_t v) { return (v + 255) / 256 * 256; }
 size_t carve(const ChebPlan& p, int N, char* base, Scratch* S) {
@@ -793,7 +805,8 @@ size_t carve(const ChebPlan& p, int N, char* base, Scratch* S) {
   S->d = reinterpret_cast<double*>(take((size_t)p.n * sizeof(double)));
   S->d_df = reinterpret_cast<float2*>(take((size_t)p.n * sizeof(float2)));
   S->report = reinterpret_cast<double*>(take(2 * sizeof(double)));
-  S->maxbits = reinterpret_cast<unsigned*>(take(sizeof(unsigned)));
+  S->maxbits = reinterpret_cast<unsigned*>(take(2 * sizeof(unsigned)));
+  S->declined = S->maxbits + 1;
   return o;
 }
 
@@ -836,19 +849,20 @@ Geom<T> make_geom(const KrylovSettings* k, double tau, const ChebPlan& p) {
   return G;
 }
 
+// slot: 0 and 1 for a call's first and second input, of which either declines.
 template <typename T>
 cudaError_t init(const Geom<T>& G, const KrylovSettings* k, const void* in, int adjoint, T* F, T* bK, const T* dK,
-                 const Scratch& S, int nset, cudaStream_t s, int64_t* launches) {
-  cudaError_t e = cudaMemsetAsync(S.maxbits, 0, sizeof(unsigned), s);
+                 const Scratch& S, int nset, int slot, cudaStream_t s, int64_t* launches) {
+  cudaError_t e = cudaMemsetAsync(S.maxbits, 0, (slot == 0 ? 2 : 1) * sizeof(unsigned), s);
   if (e != cudaSuccess) return e;
   cheb_init<T><<<dim3((unsigned)((3 * G.nk + 255) / 256), nset), 256, 0, s>>>(
       G, static_cast<const double2*>(in), k->w64, adjoint, F, bK, dK, S.maxbits);
   ++*launches;
   return cudaGetLastError();
 }
-cudaError_t report(KrylovSettings* k, const ChebPlan& p, const Scratch& S, int slot, cudaStream_t s,
+cudaError_t report(KrylovSettings* k, const ChebPlan& p, const Scratch& S, int df, int slot, cudaStream_t s,
                    int64_t* launches) {
-  cheb_report<<<1, 32, 0, s>>>(S.d, p.K, p.n, S.maxbits, S.report);
+  cheb_report<<<1, 32, 0, s>>>(S.d, p.K, p.n, S.maxbits, k->rtol, df ? 64 : 900, S.report, S.declined);
   ++*launches;
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess)
@@ -856,20 +870,22 @@ cudaError_t report(KrylovSettings* k, const ChebPlan& p, const Scratch& S, int s
   if (e == cudaSuccess) e = cudaEventRecord(k->ev[slot], s);
   return e;
 }
-// Whether the expansion stands: tail within rtol, and the input zero or of a
-// size that the arithmetic holds with room on both sides (exponents of +-64 for
-// double-float, +-900 for FP64).  Other input, NaN and infinities included, is
-// left to the Lanczos form, which normalises its vectors and reports what is
-// not finite.
-cudaError_t accepted(KrylovSettings* k, int df, int slot, bool* ok, double* bound) {
+cudaError_t accepted(KrylovSettings* k, int slot, bool* ok, double* bound) {
   const cudaError_t e = cudaEventSynchronize(k->ev[slot]);
   if (e != cudaSuccess) return e;
-  const double tail = k->pinned[2 * slot];
-  const unsigned hi = (unsigned)k->pinned[2 * slot + 1];
-  const int room = df ? 64 : 900, ex = (int)(hi >> 20) - 1023;
-  *ok = tail <= k->rtol && (hi == 0u || (ex >= -room && ex <= room));
-  *bound = std::max(*bound, tail);
+  *ok = k->pinned[2 * slot + 1] != 0.0;
+  *bound = std::max(*bound, k->pinned[2 * slot]);
   return cudaSuccess;
+}
+// Whether the input of a slot up to `slot` is declined, asked before the step that
+// follows kAhead launches of one step each: enough of them that the stream does not
+// run dry while the host learns it, and all that declined input costs.
+constexpr int kAhead = 16;
+bool known_declined(KrylovSettings* k, int slot, int launched) {
+  if (launched != kAhead) return false;
+  for (int i = 0; i <= slot; ++i)
+    if (cudaEventSynchronize(k->ev[i]) == cudaSuccess && k->pinned[2 * i + 1] == 0.0) return true;
+  return false;
 }
 rexi_status failed(cudaError_t e) {
   set_last_error(cudaGetErrorString(e));
@@ -877,13 +893,16 @@ rexi_status failed(cudaError_t e) {
 }
 
 // The Clenshaw steps k = K - 1 .. 1 on F with b_K in bA; the two newest
-// vectors are left in *b1 (b_1) and *b2 (b_2, null when K = 1).
+// vectors are left in *b1 (b_1) and *b2 (b_2, null when K = 1).  The number of
+// steps launched: fewer where the input is declined.
 template <typename T, int MODE>
-void clenshaw(const Geom<T>& G, StepArgs<T> A, int K, const T* d, T* bA, T* bB, const T* sfield, int nset,
-              cudaStream_t s, const T** b1, const T** b2) {
+int clenshaw(const Geom<T>& G, StepArgs<T> A, KrylovSettings* ks, int slot, int K, const T* d, T* bA, T* bB,
+             const T* sfield, int nset, cudaStream_t s, const T** b1, const T** b2) {
   T *cur = bA, *old = bB;
   bool have_old = false;
-  for (int k = K - 1; k >= 1; --k) {
+  int n = 0;
+  for (int k = K - 1; k >= 1; --k, ++n) {
+    if (known_declined(ks, slot, n)) break;
     A.b1 = cur;
     A.b2 = have_old ? old : nullptr;
     A.bout = old;
@@ -896,6 +915,7 @@ void clenshaw(const Geom<T>& G, StepArgs<T> A, int K, const T* d, T* bA, T* bB, 
   }
   *b1 = cur;
   *b2 = have_old ? old : nullptr;
+  return n;
 }
 
 template <typename T>
@@ -906,7 +926,7 @@ rexi_status step_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
     if (hooks.mark) hooks.mark(hooks.ctx, i, s);
   };
   int64_t launches = 0;
-  const int nset = real_input ? 1 : 2;
+  const int nset = real_input ? 1 : 2, df = std::is_same<T, double>::value ? 0 : 1;
   const Geom<T> G = make_geom<T>(k, adjoint ? -dt : dt, p);
   Scratch S;
   carve(p, M + kL, static_cast<char*>(b.scratch), &S);
@@ -915,8 +935,8 @@ rexi_status step_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
   mark(0);
   cudaError_t e = coefficients(p, h, M, S, s, &launches);
   mark(1);
-  if (e == cudaSuccess) e = init(G, k, in, adjoint ? 1 : 0, F, bA, d + p.K, S, nset, s, &launches);
-  if (e == cudaSuccess) e = report(k, p, S, 0, s, &launches);
+  if (e == cudaSuccess) e = init(G, k, in, adjoint ? 1 : 0, F, bA, d + p.K, S, nset, 0, s, &launches);
+  if (e == cudaSuccess) e = report(k, p, S, df, 0, s, &launches);
   if (e != cudaSuccess) return failed(e);
   StepArgs<T> A = {};
   A.F = F;
@@ -934,6 +954,7 @@ rexi_status step_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
     Q.H = A.H;
     Q.d = d + p.K - 1;
     Q.steps = p.K - 1;
+    Q.declined = S.declined;
     if (e == cudaSuccess) e = launch_many<T, kSum>(G, Q, mp, nset, s, &many);
     if (e != cudaSuccess) return failed(e);
     b1 = bA;
@@ -943,15 +964,14 @@ rexi_status step_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
   }
   if (!many) {
     A.bad = nullptr;
-    clenshaw<T, kSum>(G, A, p.K, d, bA, bB, nullptr, nset, s, &b1, &b2);
-    launches += p.K - 1;
+    launches += clenshaw<T, kSum>(G, A, k, 0, p.K, d, bA, bB, nullptr, nset, s, &b1, &b2);
   }
   mark(2);
   mark(3);
   // the host looks at the tail and the input while the steps run; `out` is
   // written by the last step only
   bool ok = false;
-  e = accepted(k, std::is_same<T, float2>::value, 0, &ok, bound);
+  e = accepted(k, 0, &ok, bound);
   if (e != cudaSuccess) return failed(e);
   if (ok) {
     A.b1 = b1;
@@ -993,17 +1013,19 @@ rexi_status grad_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
   ManyArgs<T> Q = {};
   Q.H = depth_table(k, T{});
   Q.steps = p.K - 1;
+  Q.declined = S.declined;
   if (many && e == cudaSuccess) e = exchange_at(mp, k, 1, b.exchange, &Q.X, s);
   // forward: P_0 in bA, P_1 in bB, then each P_{k+1} over P_{k-1}; s_k for k < K
   Geom<T> G = make_geom<T>(k, dt, p);
-  if (e == cudaSuccess) e = init(G, k, f_in, 0, bA, static_cast<T*>(nullptr), d, S, 1, s, &launches);
-  if (e == cudaSuccess) e = report(k, p, S, 0, s, &launches);
+  if (e == cudaSuccess) e = init(G, k, f_in, 0, bA, static_cast<T*>(nullptr), d, S, 1, 0, s, &launches);
+  if (e == cudaSuccess) e = report(k, p, S, df, 0, s, &launches);
   if (e != cudaSuccess) return failed(e);
   {
     StepArgs<T> A = {};
     A.H = depth_table(k, T{});
     T *cur = bA, *old = bB;
     for (int j = 0; j < p.K; ++j) {
+      if (known_declined(k, 0, j)) break;
       A.b1 = cur;
       A.b2 = j ? old : nullptr;
       A.bout = old;
@@ -1027,8 +1049,8 @@ rexi_status grad_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
   }
   // backward: the Clenshaw vectors of W^{-1} G under -dt, each step taking its s_k
   G = make_geom<T>(k, -dt, p);
-  e = init(G, k, g_out, 1, F, bA, d + p.K, S, 1, s, &launches);
-  if (e == cudaSuccess) e = report(k, p, S, 1, s, &launches);
+  e = init(G, k, g_out, 1, F, bA, d + p.K, S, 1, 1, s, &launches);
+  if (e == cudaSuccess) e = report(k, p, S, df, 1, s, &launches);
   if (e != cudaSuccess) return failed(e);
   StepArgs<T> A = {};
   A.F = F;
@@ -1054,14 +1076,13 @@ rexi_status grad_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
     launches += many;
   }
   if (!many) {
-    clenshaw<T, kGrad>(G, A, p.K, d, bA, bB, sf, 1, s, &b1, &b2);
-    launches += p.K - 1;
+    launches += clenshaw<T, kGrad>(G, A, k, 1, p.K, d, bA, bB, sf, 1, s, &b1, &b2);
   }
   mark(2);
   mark(3);
   bool okf = false, okg = false;
-  e = accepted(k, df, 0, &okf, bound);
-  if (e == cudaSuccess) e = accepted(k, df, 1, &okg, bound);
+  e = accepted(k, 0, &okf, bound);
+  if (e == cudaSuccess) e = accepted(k, 1, &okg, bound);
   if (e != cudaSuccess) return failed(e);
   if (okf && okg) {
     A.first = 0;

@@ -127,3 +127,22 @@ def test_options_and_calls_left_to_the_lanczos_form(form):
     plan.set_rho(2.0 * plan.rho)
     got, info = plan.step(to_dev(torch, st), dt, want_info=True)
     assert rel_l2(got.cpu().numpy(), R.rexii_apply_sparse(A, st.ravel(), dt, 0.5, info.M).reshape(st.shape)) < tol
+
+
+def test_declined_input_stops_the_steps():
+    """Input that is left to the Lanczos form (values outside double-float's exponents), on a grid with
+    one launch per step: no more than 16 Chebyshev steps, and six launches around them, come on top of
+    the Lanczos form's launches (alone under a cap one step below the Chebyshev degree)."""
+    torch = torch_cuda()
+    nx, ny = 701, 650
+    plan = _plan(torch, nx, ny, inputs.variable_depth(nx, ny, seed=5), "mixed", rtol=1e-8)
+    dt = 200.0 / plan.rho
+    x = to_dev(torch, inputs.kminus3_field(nx, ny, seed=6))
+    _, info = plan.step(x, dt, want_info=True)
+    launches = []
+    for cap in (20000, info.krylov_iters - 1):
+        plan.set_krylov(rtol=1e-8, max_iters=cap)
+        plan.set_profiling(True)
+        assert torch.isfinite(plan.step(x * 2.0 ** -80, dt).real).all()
+        launches.append(plan.read_profile()[2])
+    assert launches[1] < launches[0] <= launches[1] + 22
