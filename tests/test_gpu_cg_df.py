@@ -77,3 +77,20 @@ def test_iteration_cap_in_double_float_leaves_the_fp64_iterations():
         assert err.value.status == rexi.REXI_ENOCONV
         launches[rtol] = plan.read_profile()[2]
     assert launches[RTOL] >= 2 * launches[1e-14]
+
+
+def test_double_float_iterations_run_and_the_check_rejects():
+    """Ordinary values take the double-float iterations alone.  Values beyond FP32's exponents leave
+    them at x = 0, which the FP64 check rejects: those launches come on top of the FP64 iterations."""
+    torch = torch_cuda()
+    nx, ny = 20, 18
+    plan = krylov_plan(torch, nx, ny, inputs.variable_depth(nx, ny, seed=5), rtol=RTOL)
+    dt = 8.0 / plan.rho
+    st = inputs.kminus3_field(nx, ny, seed=6)
+    launches = []
+    for scale in (1.0, 2.0 ** -200):
+        plan.set_profiling(True)
+        _, info = plan.step(to_dev(torch, st * scale), dt, want_info=True)
+        launches.append(plan.read_profile()[2])
+        assert info.krylov_unconverged == 0 and info.krylov_max_rel_res <= RTOL
+    assert launches[0] < launches[1]

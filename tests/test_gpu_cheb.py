@@ -146,3 +146,41 @@ def test_declined_input_stops_the_steps():
         assert torch.isfinite(plan.step(x * 2.0 ** -80, dt).real).all()
         launches.append(plan.read_profile()[2])
     assert launches[1] < launches[0] <= launches[1] + 22
+
+
+# tiles of one launch; a grid beyond shared memory; thin complex ones (two sets) whose
+# tiles' edges are too long, narrower than the tile of the other kernel
+@pytest.mark.parametrize("form", ["fp64", "mixed"])
+@pytest.mark.parametrize("nx,ny,real,tiles", [(33, 17, True, True), (70, 3, False, True), (96, 80, True, True),
+                                              (701, 650, True, False), (16384, 11, False, False),
+                                              (5, 16384, False, False)])
+def test_which_kernel_a_grid_takes(nx, ny, real, tiles, form):
+    """The launch count tells one launch for many steps from one launch per step; the
+    latter against the Lanczos form, which a bound below 1e-13 selects."""
+    torch = torch_cuda()
+    H = inputs.variable_depth(nx, ny, seed=5)
+    st = inputs.complex_random_state(nx, ny, seed=6)
+    x = to_dev(torch, st.real if real else st)
+    plan = _plan(torch, nx, ny, H, form)
+    dt = 8.0 / plan.rho
+
+    def launches(call):
+        plan.set_profiling(True)
+        out = call()
+        return out, plan.read_profile()[2]
+
+    (got, info), n = launches(lambda: plan.step(x, dt, real_input=real, want_info=True))
+    K = info.krylov_iters
+    assert n <= 6 if tiles else K <= n <= K + 5
+    if real:
+        g = to_dev(torch, inputs.complex_random_state(nx, ny, seed=7).real)
+        (gs, gd), n = launches(lambda: plan.step_backward(x, g, dt))
+        assert n <= 12 if tiles else n >= 2 * K
+    if not tiles:
+        other = _plan(torch, nx, ny, H, "fp64", rtol=9e-14)
+        tol = _tol(form, H)
+        assert rel_l2(got.cpu().numpy(), other.step(x, dt, real_input=real).cpu().numpy()) < tol
+        if real:
+            ref_gs, ref_gd = other.step_backward(x, g, dt)
+            assert rel_l2(gs.cpu().numpy(), ref_gs.cpu().numpy()) < tol
+            assert rel_l2(gd.cpu().numpy(), ref_gd.cpu().numpy()) < max(1e-9, tol)
