@@ -360,7 +360,8 @@ OrbitParams orbits_of(const InstDesc& D) {
 }
 
 // Uploads the coefficient tables, decides per instance between the cells and
-// the persistent kernel (the rule of the single-instance step), and uploads
+// the persistent kernel (the rule of the single-instance step with its launches
+// shared), and uploads
 // the cells' descriptors and block lists.
 bool build_cells(rexi_batch_s* b, const char* tab, size_t tab_bytes) {
   if (cudaMalloc(&b->d_tables, tab_bytes) != cudaSuccess ||
@@ -786,7 +787,7 @@ rexi_status rexi_batch_step(rexi_batch_t b, const void* in, void* out, int32_t r
       fs.adjoint = 0;
       fs.exact_hn = D.exact_hn;  // the instance's table: whether every h n lies on its split grid
       const float* tab = static_cast<const float*>(b->d_tables) + D.table_off * 12;
-      // the single-instance kernels: cells or term slices as rexi_step chooses them
+      // the single-instance kernels: cells where build_cells chose them, else term slices
       const OrbitParams op = orbits_of(D);
       double2* part = reinterpret_cast<double2*>(orb);
       void* fin = orb + per_instance_part_bytes(D);

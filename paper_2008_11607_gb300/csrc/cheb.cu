@@ -371,7 +371,7 @@ void launch_step(const Geom<T>& G, const StepArgs<T>& A, int nset, cudaStream_t 
 // FMA pipe before a task took two rows); below 256^2 it is the way of an edge
 // value through L2, 1.2 us.
 struct Exchange {
-  ulonglong2 *col, *row;  // [parity][set][3][strip][ny], [parity][set][3][group][nx]
+  ulonglong2* col;        // [parity][set][3][strip][ny], then rows [parity][set][3][group][nx]
   unsigned* bad;          // a wait ran out
   unsigned* host_bad;     // the same for the host (KrylovSettings::gave_up)
   int polls;              // of one wait before a warp gives up
@@ -736,7 +736,6 @@ cudaError_t exchange_at(const ManyPlan& p, const KrylovSettings* k, int nset, vo
   X->polls = k->edge_polls;
   X->bad = reinterpret_cast<unsigned*>(b);
   X->col = reinterpret_cast<ulonglong2*>(b + 256);
-  X->row = X->col + (size_t)2 * nset * 3 * p.ns * ny;
   return cudaMemsetAsync(b, 0, exchange_bytes(p.ns, p.ng, nx, ny, nset), s);
 }
 template <typename T, int MODE>
@@ -1119,10 +1118,12 @@ rexi_status grad_impl(KrylovSettings* k, const ChebPlan& p, double h, int M, con
 // with the Lanczos form.
 bool cheb_plan(const KrylovSettings* k, double h, int M, double dt, double target, ChebPlan* p) {
   if (!(k->rho_op > 0.0)) return false;
-  // 2 / rho cut to 12 bits (the interval grows by 5e-4 at most): on unit-square
-  // grids the scaled stencil's constants are then exact in double-float too, and
-  // a small change of the depth leaves them and the coefficients as they are
-  // (differences of nearby problems see no rounding of theirs)
+  // 2 / rho cut to 12 bits (the interval grows by 5e-4 at most): a small change of
+  // the depth then leaves the scaled stencil's constants and the coefficients as they
+  // are, and where the spacings, g and f are short binary numbers (unit-square grids of
+  // 2^m points) the constants are exact in double-float too, so that differences of
+  // nearby problems see no rounding of theirs.  On other domains the constants round to
+  // 48 bits, the same for both problems unless rho crosses a step of the 12 bits
   int ex;
   p->t2 = std::frexp(2.0 / k->rho_op, &ex);
   p->t2 = std::ldexp(std::floor(std::ldexp(p->t2, 12)), ex - 12);

@@ -534,7 +534,7 @@ static int rows_threads(int rpc, int m) { return std::min(256, std::max(64, rpc 
 
 // Rows per CTA: about 1024 values, less where that would leave SMs without a CTA
 // (64^2 FP64 step 83 -> 69 us, 360 x 250 complex 145 -> 133; columns likewise, down
-// to 2, whose 32 bytes still fill a sector).
+// to 2, whose 32 bytes still fill a sector).  kFillCtas: the GPU's multiprocessors.
 constexpr int kFillCtas = 152;
 static int rows_per_cta(int n, int nrows) {
   int r = 1;

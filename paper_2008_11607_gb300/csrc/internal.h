@@ -144,7 +144,7 @@ constexpr int kCellP = 16;   // nodes per cell
 constexpr int kCellK = 32;   // cells per coarse cell
 constexpr int kCellPC = 24;  // nodes per coarse cell
 struct CellGeom {
-  double c, w, inv_c, inv_w, inv_h, q, grid, inv_grid;  // c: half-width of a cell (a power of two), w = 2c
+  double c, w, inv_w, inv_h, q, grid, inv_grid;  // c: half-width of a cell (a power of two), w = 2c
   float q_hi, q_lo;
   int k0, ncell, ncoarse, two_level;  // cells k0 .. k0 + ncell - 1, cell k on [k w, (k + 1) w)
   int tb, te, nterms;                 // the table's terms: |n| in [tb, te), n ascending

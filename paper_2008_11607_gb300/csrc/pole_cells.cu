@@ -23,9 +23,10 @@ namespace rexi {
 namespace {
 
 static_assert(kCellP == 16 && kCellPC % 2 == 0, "cell_poly's second part");
-// Lanes per node: 8, or 32 where fewer cells than this leave a multiprocessor
-// with less than four blocks, whose chains of terms then set the time (360 x
-// 250, tau rho = 120, 121 cells x 547 terms).
+// Lanes per node: 8, or 32 up to this many cells, where a multiprocessor (152 of
+// them) has less than four blocks and their chains of terms set the time (360 x 250,
+// tau rho = 120, 121 cells x 547 terms).  Near the line: 400 cells (1024^2) 11.6 us
+// with 32 lanes, 601 cells (512 x 384, scalar) 15.4 us with 8.
 constexpr int kWideCells = 600;
 
 template <int FORM>
@@ -220,8 +221,7 @@ bool cell_geometry(int form, int norb, int nterms, int tb, int te, double h, dou
   g->c = ldexp(1.0, (int)floor(log2(a / 5.13)));
   if (!(g->c > 1e-12) || !(std::max(fabs(x_lo), fabs(x_hi)) < 1e8)) return false;
   g->w = 2.0 * g->c;
-  g->inv_c = 1.0 / g->c;
-  g->inv_w = 0.5 * g->inv_c;
+  g->inv_w = 1.0 / g->w;
   g->inv_h = 1.0 / h;
   g->q = q;
   g->q_hi = (float)q;
@@ -236,8 +236,10 @@ bool cell_geometry(int form, int norb, int nterms, int tb, int te, double h, dou
   g->k0 = (int)k0;
   g->ncell = (int)(k1 - k0) + 1;
   g->ncoarse = (g->ncell + kCellK - 1) / kCellK;
-  // Costs in term evaluations: a launch is worth about 4 us of them
-  // (shared by the instances of a batch).  The cells win as soon as the orbits
+  // Costs in term evaluations: a launch is worth about 4 us of them, a fiftieth of
+  // that per instance of a batch (the mix of 96 shares each launch; small batches
+  // gain too: two of 128^2, tau rho = 50, mixed 75 -> 52 us a step, two of 64^2 stay
+  // direct; no batch of 1 to 8 instances tried was slower).  The cells win as soon as the orbits
   // outnumber the nodes by enough to pay for the extra launches: 360 x 250,
   // tau rho = 120, mixed (22,806 orbits, 1936 nodes) 52 us direct, 22 us with
   // cells; 64^2, tau rho = 50 (561 orbits, 816 nodes) stays direct.
