@@ -44,11 +44,11 @@ UNIT = "grid-points*poles/s"
 
 # DRAM traffic per launch from ncu captures on the 2048^2 grid:
 # the combine pass of the mixed form (pole_orbit_combine_df_kernel)
-NCU_COMBINE_TRAFFIC_BYTES = 110867200 + 37490176
+NCU_COMBINE_TRAFFIC_BYTES = 110814720 + 37036288
 # the forward double-float transform of real input at 2048^2 (fft_rows_r2c_kernel
 # + fft_cols_kernel, one launch each; one-pass capture of the current
 # kernels): DRAM bytes read + written by the two launches
-NCU_FFT_FWD_TRAFFIC_BYTES = (201528832 + 66863616) + (100910080 + 42878720)
+NCU_FFT_FWD_TRAFFIC_BYTES = (201434624 + 63311616) + (100847872 + 42833152)
 
 
 def set_workload(grid, tau_rho):

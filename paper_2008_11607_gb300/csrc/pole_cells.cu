@@ -25,8 +25,8 @@ namespace {
 static_assert(kCellP == 16 && kCellPC % 2 == 0, "cell_poly's second part");
 // Lanes per node: 8, or 32 up to this many cells, where a multiprocessor (152 of
 // them) has less than four blocks and their chains of terms set the time (360 x 250,
-// tau rho = 120, 121 cells x 547 terms).  Near the line: 400 cells (1024^2) 11.6 us
-// with 32 lanes, 601 cells (512 x 384, scalar) 15.4 us with 8.
+// tau rho = 120, 121 cells x 547 terms).  Near the line: 400 cells (1024^2) 11.7 us
+// with 32 lanes, 601 cells (512 x 384, scalar) 16.6 us with 8.
 constexpr int kWideCells = 600;
 
 template <int FORM>
